@@ -80,7 +80,11 @@ extern "C" {
 #define RAD_FP32_SPLIT 1     /* FP32 bulk; FP64 retarded-time anchor every K samples */
 
 /* sincos engine of the FP32 split path */
-#define RAD_VARIANT_AUTO 0   /* autotuned (or the cached choice) */
+#define RAD_VARIANT_AUTO 0   /* with 32-sample anchors and no phase budget the block-moment
+                                kernel: per particle, chunk of 32 samples and 64
+                                frequencies, polynomials in w dphi over shared moments
+                                where w dphi is small, the special-function unit
+                                elsewhere; otherwise autotuned (or the cached choice) */
 #define RAD_VARIANT_SFU 1    /* every e^{i theta} by the special-function unit */
 #define RAD_VARIANT_MIX 2    /* some frequencies by an FMA-pipe polynomial (see reserved[1]) */
 #define RAD_VARIANT_PRECISE 3 /* the offset phase nu dphi in float-float, reduced to one
@@ -136,7 +140,8 @@ typedef struct {
 
 /* Tuning knobs; zero-initialise for the defaults.  Set before the first step. */
 typedef struct {
-    int32_t variant;       /* RAD_VARIANT_*                                  */
+    int32_t variant;       /* RAD_VARIANT_*; rad_get_options reports the engine in use,
+                              RAD_VARIANT_AUTO for the block-moment kernel   */
     int32_t anchor_K;      /* FP32 path re-anchor interval: 8, 16 or 32 samples for
                               every frequency; 0 with the automatic kernel choice
                               or a phase budget in reserved[3]: the longest of 8,

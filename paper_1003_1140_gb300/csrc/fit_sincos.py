@@ -1,4 +1,5 @@
-"""Fit the FMA-pipe e^{i theta} polynomials used by the MIX variant.
+"""Fit the polynomials of the FP32 kernels: the FMA-pipe e^{i theta} of the MIX
+variant, and the cos / sin of the block-moment kernel (fit_moment).
 
 Method (written from the mathematics, not from any library's code):
   * half-angle reduction: theta/2 = k pi + y, |y| <= pi/2 (Cody & Waite two-
@@ -70,6 +71,37 @@ def fit():
     return np.float32(S), np.float32(C)
 
 
+def fit_moment(x0, n):
+    """Magnitudes of the coefficients of cos t ~ sum_j C_j (-t^2)^j and
+    sin t ~ t sum_j S_j (-t^2)^j (n terms each) on |t| <= x0: the leading ones exactly 1,
+    each next one rounded to float32 and the rest fitted again (minimax by Lawson's
+    reweighted least squares), so that the rounding of a coefficient is made up for by
+    those after it.  Interleaved C_0, S_0, C_1, ... as the kernel's table, and the
+    maximum error of both."""
+    xs = 0.5 * x0 * (1.0 - np.cos(np.pi * (np.arange(4001) + 0.5) / 4001))
+    out, worst = [], 0.0
+    for odd, fun in ((0, np.cos), (1, np.sin)):
+        pw = [xs ** (2 * k + odd) for k in range(n)]
+        coef = [1.0]
+        for step in range(1, n):
+            r = fun(xs) - sum(c * p for c, p in zip(coef, pw))
+            B = np.stack(pw[step:], 1)
+            sc = np.abs(B).max(0)
+            w, best = np.ones(len(xs)), None
+            for _ in range(300):
+                sw = np.sqrt(w)
+                c = np.linalg.lstsq(B / sc * sw[:, None], r * sw, rcond=None)[0] / sc
+                e = np.abs(r - B @ c)
+                if best is None or e.max() < best[0]:
+                    best = (e.max(), c)
+                w *= e / e.max() + 1e-3
+                w /= w.mean()
+            coef.append(float(np.float32(best[1][0])))
+        worst = max(worst, np.abs(fun(xs) - sum(c * p for c, p in zip(coef, pw))).max())
+        out.append(np.abs(coef))
+    return np.stack(out, 1).reshape(-1).astype(np.float32), worst
+
+
 PI_HI = np.float32(np.pi)
 PI_LO = np.float32(np.pi - float(PI_HI))
 INV_PI = np.float32(1.0 / np.pi)
@@ -114,3 +146,6 @@ if __name__ == "__main__":
     print("C2, C4, C6, C8 =", ", ".join(f"{v:.9e}f" for v in C))
     print("PI_HI, PI_LO =", f"{PI_HI:.9e}f, {PI_LO:.9e}f")
     print("max |error| of e^{i theta}, |theta| <= 2000:", max_error(S, C))
+    for x0, n in ((0.85, 4), (2.5, 6)):
+        c, e = fit_moment(x0, n)
+        print(f"moments, |t| <= {x0}:", ", ".join(f"{v:.9e}f" for v in c), "max error", e)

@@ -38,7 +38,7 @@
 //   the precise phase (PM: nu dphi in float-float from a ring that carries the
 //   position offsets' lo parts, reduced to one turn before the special-function
 //   unit; for every item or per item).
-// * The trajectory ring is tile-major ([tile][slot][comp][8 particles]), so a
+// * The trajectory ring is tile-major ([tile][chunk][particle][comp][32 samples]), so a
 //   chunk of 32 samples x 10 components (11 with selector flags, 14 for the
 //   precise phase) x 8 particles is one contiguous block (its anchor positions
 //   another), staged into shared memory by bulk
@@ -131,9 +131,9 @@ constexpr int kFirstOfTile = 1, kLastOfTile = 2, kFirstOfItem = 4, kLastOfItem =
 
 template <int FT, int K, bool COH, int PM = 0>
 struct Smem32 {
-    float tbuf[2][kChunk32][PM ? kCompsPrec : kComps][kTileP];     // bulk-copy destinations
-                                                      // (producer only; a chunk fills comps rows)
-    float tanc[2][kChunk32 / K][6][kTileP];           // the chunk's anchor positions (hi, lo)
+    float tbuf[2][kTileP * (PM ? kCompsPrec : kComps) * kChunk32];   // bulk-copy destinations
+                                                      // (producer only): [particle][comp][sample]
+    float tanc[2][kChunk32 / K][kTileP][6];           // the chunk's anchor positions (hi, lo)
     float4 geo[2][kComputeWarps][kChunk32 + 1];       // V1, V2, dphi per particle and sample
     // the item's nu = w / 2 pi as float-float (hi, lo): lane l's FT values as
     // FT/4 float4 slots at nu_slot<FT>(l, j)
@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     // one chunk of the ring: 32 samples x comps components x 8 particles
     const int cstride = p.comps * kTileP;
+    const int pstride = p.comps * kChunk32;   // one particle's samples of the chunk
     const uint32_t kBytes = (uint32_t)(kChunk32 * cstride * sizeof(float));
     constexpr int kNRun = (COH ? 4 : 1) * FT * 32;
     constexpr int NS = FT - NP;   // SFU frequencies per thread
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 const float* asrc = p.anc32 + (tile * p.nblk + blk) * (6 * kTileP);
                 fence_proxy_async();
                 mbar_arrive_expect_tx(&S.tfull[buf], kBytes + kAncBytes);
-                bulk_load(&S.tbuf[buf][0][0][0], src, kBytes, &S.tfull[buf]);
+                bulk_load(&S.tbuf[buf][0], src, kBytes, &S.tfull[buf]);
                 bulk_load(&S.tanc[buf][0][0][0], asrc, kAncBytes, &S.tfull[buf]);
             }
             ++uses[buf];
@@ -354,8 +355,8 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 const float nh[3] = {n0, n1, n2}, nlo[3] = {nl0, nl1, nl2};
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    const ff dh = two_sum(S.tanc[buf][b][q][pp], -S.tanc[buf][bA][q][pp]);
-                    const float dl = dh.lo + (S.tanc[buf][b][3 + q][pp] - S.tanc[buf][bA][3 + q][pp]);
+                    const ff dh = two_sum(S.tanc[buf][b][pp][q], -S.tanc[buf][bA][pp][q]);
+                    const float dl = dh.lo + (S.tanc[buf][b][pp][3 + q] - S.tanc[buf][bA][pp][3 + q]);
                     const ff d = two_prod(nh[q], dh.hi);
                     const float dd = fmaf(nh[q], dl, fmaf(nlo[q], dh.hi, d.lo));
                     const ff u = two_sum(sh, d.hi);
@@ -384,12 +385,12 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 const int mhi = hi - 1 < bl + KE - 1 ? hi - 1 : bl + KE - 1;
                 float h = 0.5f * (float)(KE - 1) * p.dt_hi;
                 if (mlo <= mhi) {
-                    const float* t0 = &S.tbuf[buf][0][0][0] + mlo * cstride + pp;
-                    const float* t1 = &S.tbuf[buf][0][0][0] + mhi * cstride + pp;
+                    const float* t0 = &S.tbuf[buf][0] + pp * pstride + mlo;
+                    const float* t1 = &S.tbuf[buf][0] + pp * pstride + mhi;
                     float o0 = (float)(mlo - bl) * p.dt_hi -
-                               (n0 * t0[0] + n1 * t0[kTileP] + n2 * t0[2 * kTileP]);
+                               (n0 * t0[0] + n1 * t0[kChunk32] + n2 * t0[2 * kChunk32]);
                     float o1 = (float)(mhi - bl) * p.dt_hi -
-                               (n0 * t1[0] + n1 * t1[kTileP] + n2 * t1[2 * kTileP]);
+                               (n0 * t1[0] + n1 * t1[kChunk32] + n2 * t1[2 * kChunk32]);
                     if (kmul > 0) {
                         o0 -= S.cof[pp][mlo >> kLog2K].x;
                         o1 -= S.cof[pp][mhi >> kLog2K].x;
@@ -407,7 +408,7 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 const float nh[3] = {n0, n1, n2}, nlo[3] = {nl0, nl1, nl2};
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    const float rh = S.tanc[buf][bA][q][pp], rl = S.tanc[buf][bA][3 + q][pp];
+                    const float rh = S.tanc[buf][bA][pp][q], rl = S.tanc[buf][bA][pp][3 + q];
                     const ff d = two_prod(nh[q], rh);
                     const float dl = fmaf(nh[q], rl, fmaf(nlo[q], rh, d.lo));
                     const ff u = two_sum(sh, -d.hi);
@@ -418,14 +419,14 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 S.anc[buf][pp][B] = make_float2(hi, e - (hi - sh));
             }
             __syncwarp();
-            // geometry: round r handles sample 4 r + lane / 8 of particle lane % 8
+            // geometry: round r handles particle r, lane = sample
 #pragma unroll 2
-            for (int r = 0; r < kChunk32 / 4; ++r) {
-                const int sm = 4 * r + (lane >> 3), pp = lane & (kTileP - 1);
-                const float* tb = &S.tbuf[buf][0][0][0] + sm * cstride + pp;
-                const float b0 = tb[3 * kTileP], b1 = tb[4 * kTileP], b2 = tb[5 * kTileP];
-                const float d0 = tb[6 * kTileP], d1 = tb[7 * kTileP], d2 = tb[8 * kTileP];
-                const float g = tb[9 * kTileP];
+            for (int r = 0; r < kTileP; ++r) {
+                const int sm = lane, pp = r;
+                const float* tb = &S.tbuf[buf][0] + pp * pstride + sm;
+                const float b0 = tb[3 * kChunk32], b1 = tb[4 * kChunk32], b2 = tb[5 * kChunk32];
+                const float d0 = tb[6 * kChunk32], d1 = tb[7 * kChunk32], d2 = tb[8 * kChunk32];
+                const float g = tb[9 * kChunk32];
                 const float bn = n0 * b0 + n1 * b1 + n2 * b2;
                 const float p1 = e10 * b0 + e11 * b1 + e12 * b2;
                 const float p2 = e20 * b0 + e21 * b1 + e22 * b2;
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 const float inv = qdt / (kap * kap);
                 float V1 = -(p1 * dn + q1 * kap) * inv;
                 float V2 = -(p2 * dn + q2 * kap) * inv;
-                if (selb >= 0 && !((__float_as_uint(tb[10 * kTileP]) >> selb) & 1u)) V1 = V2 = 0.0f;
+                if (selb >= 0 && !((__float_as_uint(tb[10 * kChunk32]) >> selb) & 1u)) V1 = V2 = 0.0f;
                 // dphi = (sm mod KE) dt - h - n . dr (- C), compensated
                 const float ti = (float)(sm & (KE - 1));
                 const ff t = two_prod(ti, p.dt_hi);
@@ -450,13 +451,13 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                     sh = u.hi;
                     e = e + (u.lo - cf.y);
                 }
-                const float dr[3] = {tb[0], tb[kTileP], tb[2 * kTileP]};
+                const float dr[3] = {tb[0], tb[kChunk32], tb[2 * kChunk32]};
                 const float nh[3] = {n0, n1, n2}, nlo[3] = {nl0, nl1, nl2};
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     const ff d = two_prod(nh[q], dr[q]);
                     float dl = fmaf(nlo[q], dr[q], d.lo);
-                    if (PM) dl = fmaf(nh[q], tb[(11 + q) * kTileP], dl);   // n . dr_lo
+                    if (PM) dl = fmaf(nh[q], tb[(11 + q) * kChunk32], dl);   // n . dr_lo
                     const ff u = two_sum(sh, -d.hi);
                     sh = u.hi;
                     e = e + (u.lo - dl);

@@ -91,8 +91,8 @@ struct rad_ctx {
     // configuration
     int D = 0;
     int n_grids = 0;
-    std::vector<int> grid_off, grid_len;
-    std::vector<double> h_freqs;    // all frequency grids, concatenated
+    std::vector<int> grid_off, grid_len;   // offsets into the padded arrays
+    std::vector<double> h_freqs;    // all frequency grids, each padded to kFreqPad
     double dt = 0.0, box_L = 0.0;
     int mode = 0, precision = 0;
     int n_species = 0;
@@ -273,6 +273,7 @@ static void basis(const double n[3], double e1[3], double e2[3])
 bool rad::accum32_dispatch(const Accum32Params* p, const Accum32Config& cfg, int grid,
                            cudaStream_t st, cudaError_t* err, int* nb)
 {
+    if (cfg.mom) return accum32_moment(p, cfg, grid, st, err, nb);
     if (cfg.pm) return accum32_precise(p, cfg, grid, st, err, nb);
     if (cfg.band) return accum32_band(p, cfg, grid, st, err, nb);
     return accum32_ft8_sfu(p, cfg, grid, st, err, nb) || accum32_ft8_mix(p, cfg, grid, st, err, nb) ||
@@ -456,7 +457,7 @@ static std::string tune_key(const rad_ctx* c, int K)
           << c->win_dirs[w].size() << ",";
     }
     k << "|d" << c->opt.defer << "|n" << std::max(1, c->opt.subcycle) << "|b" << c->cfg.band
-      << "|p" << c->cfg.pm;
+      << "|p" << c->cfg.pm << (c->cfg.mom ? "|moments" : "");
     return k.str();
 }
 
@@ -550,9 +551,15 @@ static int autotune32(rad_ctx* c, int K)
                                         {8, 1, K, coh, 3}, {8, 2, K, coh, 2}, {4, 0, K, coh, 4}};
     if (c->cfg.band) cands = {{8, 0, K, coh, 2, true}, {8, 0, K, coh, 3, true}};
     if (c->cfg.pm) cands = {{8, 0, K, coh, 2, false, c->cfg.pm}, {8, 0, K, coh, 3, false, c->cfg.pm}};
+    if (c->cfg.mom) cands = {{8, 0, K, coh, 2, false, 0, true}};
     // small problems: not worth timing
     if (rad_updates(c) < (int64_t)2e10) {
         c->cfg = cands[0];
+        return RAD_OK;
+    }
+    if (cands.size() == 1) {         // nothing to choose from: only the record
+        c->cfg = cands[0];
+        tune_store(key, c->cfg);
         return RAD_OK;
     }
     float best_ms = 1e30f;
@@ -743,6 +750,9 @@ static int freeze(rad_ctx* c)
             c->cfg.ft = 8;
             c->cfg.np = 0;
         }
+        // the automatic engine at the 32-sample anchors is the block-moment kernel
+        c->cfg.mom = !prec && !c->cfg.band && c->opt.variant == RAD_VARIANT_AUTO && c->K == 32 &&
+                     c->opt.reserved[3] == 0 && c->cfg.ft == 8 && c->cfg.mb == 2;
         // anchor positions: one FP32 hi/lo 3-vector per particle per K samples of the ring
         c->nblk = c->ring / c->K;
         if (!c->anc32) {
@@ -885,11 +895,15 @@ static IngestParams ingest_params(const rad_ctx* c)
 }
 
 // Scratch of a time-segmented ingest launch over count particles and n_steps
-// calls (segments of kSegLen calls, a multiple of every anchor interval).
+// calls: segments of whole 32-sample chunks, or of kSegLen calls (a multiple of every
+// anchor interval) with sub-cycling; none where launch_ingest does not split.
 constexpr int kSegLen = 64;
 static int seg_scratch(rad_ctx* c, int64_t count, int64_t n_steps, IngestParams& p)
 {
-    const int64_t nseg_max = std::min<int64_t>(n_steps / kSegLen + 2, 257);   // launch_ingest caps at 256
+    p.state_out = nullptr;
+    p.wind = nullptr;
+    if (count >= (c->nsub > 1 ? kSegMaxParticles : (int64_t)kSegMaxTiles * kTileP)) return RAD_OK;
+    const int64_t nseg_max = std::min<int64_t>(n_steps / kChunk32 + 2, 257);   // launch_ingest caps at 256
     const size_t sb = (size_t)9 * count * sizeof(double);
     const size_t wb = (size_t)nseg_max * 3 * count * sizeof(int32_t);
     if (c->seg_bytes < sb + wb) {
@@ -1320,11 +1334,17 @@ int rad_init(rad_ctx** out, const double* dirs, int32_t D, const double* freqs,
         if (grid_len[g] < 1) return bail(RAD_EINVAL);
         c->grid_off.push_back((int)nf);
         c->grid_len.push_back(grid_len[g]);
-        nf += grid_len[g];
+        nf += ((int64_t)grid_len[g] + kFreqPad - 1) / kFreqPad * kFreqPad;
     }
-    for (int64_t i = 0; i < nf; ++i)
-        if (!std::isfinite(freqs[i])) return bail(RAD_EINVAL);
-    c->h_freqs.assign(freqs, freqs + nf);
+    c->h_freqs.assign(nf, 0.0);
+    {
+        int64_t k = 0;
+        for (int g = 0; g < n_grids; ++g)
+            for (int i = 0; i < grid_len[g]; ++i, ++k) {
+                if (!std::isfinite(freqs[k])) return bail(RAD_EINVAL);
+                c->h_freqs[c->grid_off[g] + i] = freqs[k];
+            }
+    }
     c->in_off.push_back(0);
     int64_t col = 0;
     for (int s = 0; s < n_species; ++s) {
@@ -1408,8 +1428,8 @@ int rad_init(rad_ctx** out, const double* dirs, int32_t D, const double* freqs,
     std::vector<float> om32(nf), nuh(nf), nul(nf);
     const double two_pi = 6.283185307179586476925286766559;
     for (int64_t i = 0; i < nf; ++i) {
-        om32[i] = (float)freqs[i];
-        const double nu = freqs[i] / two_pi;
+        om32[i] = (float)c->h_freqs[i];
+        const double nu = c->h_freqs[i] / two_pi;
         nuh[i] = (float)nu;
         nul[i] = (float)(nu - (double)nuh[i]);
     }
@@ -1443,7 +1463,7 @@ int rad_init(rad_ctx** out, const double* dirs, int32_t D, const double* freqs,
     CUB(cudaMemcpy(c->d_om32, om32.data(), nf * sizeof(float), cudaMemcpyHostToDevice));
     CUB(cudaMemcpy(c->d_nuhi, nuh.data(), nf * sizeof(float), cudaMemcpyHostToDevice));
     CUB(cudaMemcpy(c->d_nulo, nul.data(), nf * sizeof(float), cudaMemcpyHostToDevice));
-    CUB(cudaMemcpy(c->d_om64, freqs, nf * sizeof(double), cudaMemcpyHostToDevice));
+    CUB(cudaMemcpy(c->d_om64, c->h_freqs.data(), nf * sizeof(double), cudaMemcpyHostToDevice));
     CUB(cudaMemcpy(c->d_wins, wd.data(), n_win * sizeof(WinDev), cudaMemcpyHostToDevice));
     CUB(cudaMemcpy(c->d_species, sd.data(), n_species * sizeof(SpeciesDev), cudaMemcpyHostToDevice));
 
@@ -1577,7 +1597,8 @@ int rad_get_options(const rad_ctx* c, rad_options* o)
         o->freq_per_lane = c->cfg.ft;
         o->blocks_per_sm = c->cfg.mb;
         o->variant = c->cfg.pm ? RAD_VARIANT_PRECISE
-                                 : (c->cfg.np > 0 ? RAD_VARIANT_MIX : RAD_VARIANT_SFU);
+                     : c->cfg.mom ? RAD_VARIANT_AUTO
+                                  : (c->cfg.np > 0 ? RAD_VARIANT_MIX : RAD_VARIANT_SFU);
         o->reserved[1] = c->cfg.np;
     }
     return RAD_OK;

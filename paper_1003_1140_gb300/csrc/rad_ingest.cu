@@ -7,13 +7,19 @@
 //   beta_m    = ubar / sqrt(1 + ubar^2),  ubar = (u_{m-1/2} + u_{m+1/2}) / 2,
 //   betadot_m = (beta_{m+1/2} - beta_{m-1/2}) / dt,
 //   g_m       = 1/gamma_m^2 = 1 / (1 + ubar^2).
-// A thread walks one particle through one time segment of the launch's steps,
-// keeping the previous raw position, the image count n (the unwrapped position
-// is r = x + L n) and u_{s-3/2} in registers; the per-particle state arrays
-// carry them between launches.  Segments after the first start at
-// anchor-aligned samples; their starting image count is the launch's initial
-// count plus the integer changes of the earlier segments (wind_kernel), so the
-// split in time changes no result.
+// The per-particle state arrays carry the previous raw position, the image count n
+// (the unwrapped position is r = x + L n) and u_{s-1/2} between launches.  Two
+// kernels:
+//   * ingest_tile_kernel (batches of calls): a block turns chunks of 32 samples of one
+//     8-particle tile into ring records, one thread per sample, and writes each
+//     record as one contiguous block;
+//   * ingest_kernel (a few calls, or sub-cycling): a thread walks one particle
+//     through one time segment of the launch's steps.
+// Both split a launch in time when the particles alone leave the GPU idle: a later
+// segment's starting image count is the launch's initial count plus the integer
+// changes of the earlier segments (wind kernels), so the split changes no result.
+#include <algorithm>
+
 #include "rad_internal.cuh"
 
 namespace rad {
@@ -104,6 +110,13 @@ __device__ uint32_t selector_bits(const IngestParams& p, const double x[3], cons
         bits |= (in ? 1u : 0u) << i;
     }
     return bits;
+}
+
+// Component 0 of a sample in the FP32 ring (components are kChunk32 apart).
+__device__ __forceinline__ float* slab32_at(const IngestParams& p, int64_t tile, int64_t slot, int64_t pp)
+{
+    return p.slab32 + (((tile * p.ring + slot) / kChunk32 * kTileP + pp) * p.comps) * kChunk32 +
+           slot % kChunk32;
 }
 
 // 64-thread blocks (launch_ingest), at least 8 resident per SM: the FP64-bound
@@ -247,33 +260,33 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                 const int64_t M = m * p.nsub + k;
                 const int64_t sl = M % p.ring;
                 if (p.slab32) {
-                    float* an = p.anc32 + (tile * p.nblk + (M / p.K) % p.nblk) * (6 * kTileP) + pp;
+                    float* an = p.anc32 + ((tile * p.nblk + (M / p.K) % p.nblk) * kTileP + pp) * 6;
                     if ((M % p.K) == 0 || !have_anchor) {
                         if ((M % p.K) == 0) {
                             for (int c = 0; c < 3; ++c) {
                                 const float hi = (float)rk[c];
                                 const float lo = (float)(rk[c] - (double)hi);
-                                an[c * kTileP] = hi;
-                                an[(3 + c) * kTileP] = lo;
+                                an[c] = hi;
+                                an[3 + c] = lo;
                                 ra[c] = (double)hi + (double)lo;
                             }
                         } else {
                             for (int c = 0; c < 3; ++c)
-                                ra[c] = (double)an[c * kTileP] + (double)an[(3 + c) * kTileP];
+                                ra[c] = (double)an[c] + (double)an[3 + c];
                         }
                         have_anchor = true;
                     }
-                    float* o = p.slab32 + (tile * p.ring + sl) * (p.comps * kTileP) + pp;
+                    float* o = slab32_at(p, tile, sl, pp);
                     for (int c = 0; c < 3; ++c) {
                         const double d = rk[c] - ra[c];
                         const float dh = (float)d;
-                        o[c * kTileP] = dh;
-                        if (PRING) o[(11 + c) * kTileP] = (float)(d - (double)dh);
-                        o[(3 + c) * kTileP] = (float)bk[c];
-                        o[(6 + c) * kTileP] = (float)bd[c];
+                        o[c * kChunk32] = dh;
+                        if (PRING) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
+                        o[(3 + c) * kChunk32] = (float)bk[c];
+                        o[(6 + c) * kChunk32] = (float)bd[c];
                     }
-                    o[9 * kTileP] = (float)(1.0 / gk2);
-                    if (p.comps > kCompsPlain) o[10 * kTileP] = __uint_as_float(flags);
+                    o[9 * kChunk32] = (float)(1.0 / gk2);
+                    if (p.comps > kCompsPlain) o[10 * kChunk32] = __uint_as_float(flags);
                 } else {
                     double* o = p.slab64 + (tile * p.ring + sl) * (p.comps * kTileP) + pp;
                     for (int c = 0; c < 3; ++c) {
@@ -294,18 +307,18 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             // and weakly parallel accelerations a frozen-field push produces.
             // anchor position r_a as an FP32 hi + lo pair; dr is taken relative
             // to exactly hi + lo, the value the accumulation kernel sees
-            float* an = p.anc32 + (tile * p.nblk + blk) * (6 * kTileP) + pp;
+            float* an = p.anc32 + ((tile * p.nblk + blk) * kTileP + pp) * 6;
             if (kpos == 0) {
                 for (int c = 0; c < 3; ++c) {
                     const float hi = (float)rp[c];
                     const float lo = (float)(rp[c] - (double)hi);
-                    an[c * kTileP] = hi;
-                    an[(3 + c) * kTileP] = lo;
+                    an[c] = hi;
+                    an[3 + c] = lo;
                     ra[c] = (double)hi + (double)lo;
                 }
                 have_anchor = true;
             } else if (!have_anchor) {
-                for (int c = 0; c < 3; ++c) ra[c] = (double)an[c * kTileP] + (double)an[(3 + c) * kTileP];
+                for (int c = 0; c < 3; ++c) ra[c] = (double)an[c] + (double)an[3 + c];
                 have_anchor = true;
             }
             float um[3], uq[3], du[3], ub[3];
@@ -324,26 +337,26 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             const float igq = 1.0f / gq;
             const float corr = dus / (gq * gm * (gq + gm));
             const float idt = (float)(1.0 / p.dt);
-            float* o = p.slab32 + (tile * p.ring + slot) * (p.comps * kTileP) + pp;
+            float* o = slab32_at(p, tile, slot, pp);
             for (int c = 0; c < 3; ++c) {
                 const double d = rp[c] - ra[c];
                 const float dh = (float)d;
-                o[c * kTileP] = dh;
+                o[c * kChunk32] = dh;
                 // precise-phase ring: the rounding of the offset as its lo part
-                if (PRING) o[(11 + c) * kTileP] = (float)(d - (double)dh);
+                if (PRING) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
             }
-            o[3 * kTileP] = ub[0] * igb;
-            o[4 * kTileP] = ub[1] * igb;
-            o[5 * kTileP] = ub[2] * igb;
-            o[6 * kTileP] = (du[0] * igq - um[0] * corr) * idt;
-            o[7 * kTileP] = (du[1] * igq - um[1] * corr) * idt;
-            o[8 * kTileP] = (du[2] * igq - um[2] * corr) * idt;
-            o[9 * kTileP] = 1.0f / gb2;
+            o[3 * kChunk32] = ub[0] * igb;
+            o[4 * kChunk32] = ub[1] * igb;
+            o[5 * kChunk32] = ub[2] * igb;
+            o[6 * kChunk32] = (du[0] * igq - um[0] * corr) * idt;
+            o[7 * kChunk32] = (du[1] * igq - um[1] * corr) * idt;
+            o[8 * kChunk32] = (du[2] * igq - um[2] * corr) * idt;
+            o[9 * kChunk32] = 1.0f / gb2;
             if (p.comps > kCompsPlain) {
                 double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
                                  __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
                                  __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
-                o[10 * kTileP] = __uint_as_float(p.n_sel ? selector_bits(p, xp, ubd) : 0xffffffffu);
+                o[10 * kChunk32] = __uint_as_float(p.n_sel ? selector_bits(p, xp, ubd) : 0xffffffffu);
             }
         } else {
             double ub[3];
@@ -410,10 +423,356 @@ __global__ void store_state(const IngestParams p)
     }
 }
 
+// The binary exponent and leading 20 mantissa bits of a double as a float (truncated;
+// magnitudes below the float range become 0, above it infinity): integer work only.
+__device__ __forceinline__ float coarse(double v)
+{
+    const int hi = __double2hiint(v);
+    const int t = (hi & 0x7fffffff) - (896 << 20);
+    const uint32_t m = t <= 0 ? 0u : (t >= (255 << 20) ? 0x7f800000u : (uint32_t)t << 3);
+    return __uint_as_float(m | ((uint32_t)hi & 0x80000000u));
+}
+
+// False only if the displacement b - a is surely within half a box (no crossing): the
+// difference of the coarse values plus their truncation (2^-20 of each) against
+// 0.4999 L.  Keeps the 1/64-rate FP64 pipe out of the common case.
+__device__ __forceinline__ bool maybe_jump(double a, double b, float lim)
+{
+    const float fa = coarse(a), fb = coarse(b);
+    return !(fmaf(fmaxf(fabsf(fa), fabsf(fb)), 1.9073486e-6f, fabsf(fb - fa)) <= lim);
+}
+
+// Geometry of a batched launch: samples [m0, m1], chunks [c0, c1], calls up to s1.
+struct BatchRange {
+    int64_t m0, m1, s1, c0, c1;
+};
+__host__ __device__ __forceinline__ BatchRange batch_range(const IngestParams& p)
+{
+    BatchRange b;
+    b.m0 = p.step0 > 0 ? p.step0 - 1 : 0;
+    b.s1 = p.step0 + p.n_steps - 1;
+    b.m1 = b.s1 - 1;
+    b.c0 = b.m0 / kChunk32;
+    b.c1 = b.m1 / kChunk32;
+    return b;
+}
+
+// Particle of tile column col: its species' input index, or -1 (padding, or outside
+// the launch's particle range).
+__device__ __forceinline__ int64_t tile_particle(const IngestParams& p, int64_t col)
+{
+    int sp = 0;
+    while (sp + 1 < p.n_species &&
+           (col >= p.col_off[sp + 1] || p.in_off[sp + 1] == p.in_off[sp]))
+        ++sp;
+    const int64_t i = p.in_off[sp] + (col - p.col_off[sp]);
+    const int64_t end = p.count ? p.first + p.count : p.n_in;
+    return col >= p.col_off[sp] && i < p.in_off[sp + 1] && i >= p.first && i < end ? i : -1;
+}
+
+// Change of the image count over each segment but the last of a batched launch
+// (box_L > 0): one thread per particle and segment, eight calls' loads in flight.
+__global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
+{
+    const int64_t cnt = p.count ? p.count : p.n_in - p.first;
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= cnt * (p.n_seg - 1)) return;
+    const int g = (int)(q / cnt);
+    const int64_t k = q - (int64_t)g * cnt, i = p.first + k;
+    const int64_t ld = p.ld ? p.ld : p.n_in, xi = i - p.xoff;
+    const BatchRange b = batch_range(p);
+    // calls (sa, sb] of the segment's samples
+    const int64_t sa = g == 0 ? b.m0 : (b.c0 + (int64_t)g * p.seg_len) * kChunk32;
+    const int64_t sb = (b.c0 + (int64_t)(g + 1) * p.seg_len) * kChunk32;
+    const float lim = 0.4999f * (float)p.box_L;
+    const double half_L = 0.5 * p.box_L;
+    const double* x = p.x + xi;
+    double xp[3];
+    int32_t dn[3] = {0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (sa >= p.step0) {
+            xp[c] = x[((sa - p.step0) * 3 + c) * ld];
+        } else {
+            int sp = 0;
+            while (sp + 1 < p.n_species && i >= p.in_off[sp + 1]) ++sp;
+            xp[c] = p.x_prev[c * p.ncols + p.col_off[sp] + (i - p.in_off[sp])];
+        }
+    }
+    constexpr int U = 8;
+    for (int64_t s = sa + 1; s <= sb; s += U) {
+        double xn[U][3];
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                xn[j][c] = x[((min(s + j, sb) - p.step0) * 3 + c) * ld];
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (maybe_jump(xp[c], xn[j][c], lim))
+                    dn[c] -= (int32_t)image_jump(xn[j][c] - xp[c], p.box_L, half_L);
+                xp[c] = xn[j][c];
+            }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) p.wind[((int64_t)g * 3 + c) * cnt + k] = dn[c];
+}
+
+// One block: chunks [q0, q1) (32 samples each) of one 8-particle tile, thread = sample
+// and particle.  Rows of 33 calls go through shared memory (a sample needs u of two
+// calls); the image counts change only at a crossing, found with integer and FP32
+// work, so the FP64 work per sample is one subtraction and two conversions per
+// component of x and u (the previous kernel, one thread per particle for every call,
+// ran 27 FP64 instructions per sample and a serial chain over the calls: 192 us for
+// 1024 particles x 2000 calls).  The record of a chunk is staged in shared memory and
+// written as one contiguous block.  MODE 0: FP32 ring, 1: the precise-phase FP32 ring
+// (the offsets' lo part too), 2: FP64 ring (its 16-sample chunks have the same order of
+// slots; samples are written directly).
+template <int MODE>
+__global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(const IngestParams p)
+{
+    __shared__ double xs[kChunk32 + 1][3][kTileP], us[kChunk32 + 1][3][kTileP];
+    __shared__ double ras[kChunk32 / 8][3][kTileP];
+    __shared__ int cnt[3][kTileP], moved[3][kTileP];
+    extern __shared__ __align__(16) float outs[];       // [particle][comp][sample], padded
+    int(*jc)[3][kTileP] = reinterpret_cast<int(*)[3][kTileP]>(outs);
+    const int tid = threadIdx.x, sm = tid >> 3, pp = tid & (kTileP - 1);
+    const int tile_l = (int)(blockIdx.x % p.n_tiles), g = (int)(blockIdx.x / p.n_tiles);
+    const int64_t tile = p.tile0 + tile_l, col = tile * kTileP + pp;
+    const int64_t i = tile_particle(p, col);
+    const int64_t npart = p.count ? p.count : p.n_in - p.first;
+    const int64_t ld = p.ld ? p.ld : p.n_in, xi = i - p.xoff;
+    const BatchRange b = batch_range(p);
+    const int64_t q0 = b.c0 + (int64_t)g * p.seg_len;
+    const int64_t q1 = min(q0 + p.seg_len, b.c1 + 1);
+    const bool box = p.box_L > 0.0;
+    const float lim = 0.4999f * (float)p.box_L;
+    const float idt = (float)(1.0 / p.dt);
+    const int ostride = p.comps * kChunk32 + 4;
+    bool bad = false;
+
+    if (tid < 3 * kTileP) {
+        const int c = tid >> 3;
+        int n = 0;
+        if (box && i >= 0) {
+            if (p.step0 > 0) n = (int)p.r_prev[c * p.ncols + col];
+            for (int h = 0; h < g; ++h) n += p.wind[((int64_t)h * 3 + c) * npart + (i - p.first)];
+        }
+        cnt[c][pp] = n;
+    }
+    auto row = [&](int64_t s, int r, int c) {            // one value each of x and u
+        double xv = 0.0, uv = 0.0;
+        if (i >= 0 && s >= b.m0 && s <= b.s1) {
+            if (s >= p.step0) {
+                xv = p.x[((s - p.step0) * 3 + c) * ld + xi];
+                uv = p.u[((s - p.step0) * 3 + c) * ld + xi];
+                if (p.check) bad |= !isfinite(xv) || !isfinite(uv);
+            } else {
+                xv = p.x_prev[c * p.ncols + col];
+                uv = p.u_prev[c * p.ncols + col];
+            }
+        }
+        xs[r][c][pp] = xv;
+        us[r][c][pp] = uv;
+    };
+    uint32_t rc = (uint32_t)(q0 % (p.ring / kChunk32));  // ring chunk of chunk q
+    for (int64_t q = q0; q < q1; ++q) {
+        const int64_t m = q * kChunk32 + sm, slot0 = (int64_t)rc * kChunk32;
+        if (++rc == (uint32_t)(p.ring / kChunk32)) rc = 0;
+        const bool valid = m >= b.m0 && m <= b.m1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) row(m, sm, c);
+        if (tid < 3 * kTileP) row(q * kChunk32 + kChunk32, kChunk32, tid >> 3);
+        __syncthreads();
+        double x[3], up[3], un[3];
+        bool jump = false;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            x[c] = xs[sm][c][pp];
+            up[c] = us[sm][c][pp];
+            un[c] = us[sm + 1][c][pp];
+            jump |= box && valid && maybe_jump(x[c], xs[sm + 1][c][pp], lim);
+        }
+        // image counts: the chunk's starting count unless something crossed in it
+        const bool any = __syncthreads_or(jump);
+        int n[3] = {cnt[0][pp], cnt[1][pp], cnt[2][pp]};
+        if (any) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                jc[sm][c][pp] =
+                    jump ? (int)image_jump(xs[sm + 1][c][pp] - x[c], p.box_L, 0.5 * p.box_L) : 0;
+            __syncthreads();
+            for (int r = 0; r < sm; ++r)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) n[c] -= jc[r][c][pp];
+        }
+        // anchors: r_a as an FP32 hi + lo pair; offsets are relative to exactly hi + lo
+        if (MODE != 2 && sm % p.K == 0) {
+            float* an = p.anc32 + ((tile * p.nblk + (slot0 + sm) / p.K) * kTileP + pp) * 6;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float hi = 0.0f, lo = 0.0f;
+                if (valid && i >= 0) {
+                    const double r = x[c] + p.box_L * (double)n[c];
+                    hi = (float)r;
+                    lo = (float)(r - (double)hi);
+                    an[c] = hi;
+                    an[3 + c] = lo;
+                } else if (i >= 0 && m < b.m0) {         // written by an earlier launch
+                    hi = an[c];
+                    lo = an[3 + c];
+                }
+                const double ra = (double)hi + (double)lo;
+                ras[sm / p.K][c][pp] = any ? ra : ra - p.box_L * (double)n[c];
+            }
+        }
+        __syncthreads();                                 // ras; jc read by everyone
+        if (any && tid < 3 * kTileP) {
+            int t = 0;
+            for (int r = 0; r < kChunk32; ++r) t += jc[r][tid >> 3][pp];
+            moved[tid >> 3][pp] = t;                     // zero beyond the last call
+        }
+        if (any) __syncthreads();
+        if (MODE == 2) {
+            if (valid && i >= 0) {
+                double ub[3];
+                for (int c = 0; c < 3; ++c) ub[c] = 0.5 * (up[c] + un[c]);
+                const double gm = sqrt(1.0 + (up[0] * up[0] + up[1] * up[1] + up[2] * up[2]));
+                const double gp = sqrt(1.0 + (un[0] * un[0] + un[1] * un[1] + un[2] * un[2]));
+                const double gb2 = 1.0 + (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
+                const double gb = sqrt(gb2);
+                double* o = p.slab64 + (tile * p.ring + slot0 + sm) * (p.comps * kTileP) + pp;
+                for (int c = 0; c < 3; ++c) {
+                    o[c * kTileP] = x[c] + p.box_L * (double)n[c];
+                    o[(3 + c) * kTileP] = ub[c] / gb;
+                    o[(6 + c) * kTileP] = (un[c] / gp - up[c] / gm) / p.dt;
+                }
+                o[9 * kTileP] = 1.0 / gb2;
+                if (p.comps > kCompsPlain) {
+                    double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
+                                     __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
+                                     __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
+                    o[10 * kTileP] = (double)(p.n_sel ? selector_bits(p, x, ubd) : 0xffffffffu);
+                }
+            }
+        } else {
+            // as ingest_kernel: only the cancellation-prone differences in FP64
+            float* o = outs + pp * ostride + sm;
+            float um[3], uq[3], du[3], ub[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const double ra = ras[sm / p.K][c][pp];
+                const double d = any ? (x[c] + p.box_L * (double)n[c]) - ra : x[c] - ra;
+                const float dh = (float)d;
+                o[c * kChunk32] = dh;
+                if (MODE == 1) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
+                um[c] = (float)up[c];
+                uq[c] = (float)un[c];
+                du[c] = (float)(un[c] - up[c]);
+                ub[c] = 0.5f * (um[c] + uq[c]);
+            }
+            const float gm = sqrtf(1.0f + (um[0] * um[0] + um[1] * um[1] + um[2] * um[2]));
+            const float gq = sqrtf(1.0f + (uq[0] * uq[0] + uq[1] * uq[1] + uq[2] * uq[2]));
+            const float gb2 = 1.0f + (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
+            const float igb = rsqrtf(gb2);
+            const float dus = du[0] * (uq[0] + um[0]) + du[1] * (uq[1] + um[1]) +
+                              du[2] * (uq[2] + um[2]);
+            const float igq = 1.0f / gq;
+            const float corr = dus / (gq * gm * (gq + gm));
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                o[(3 + c) * kChunk32] = ub[c] * igb;
+                o[(6 + c) * kChunk32] = (du[c] * igq - um[c] * corr) * idt;
+            }
+            o[9 * kChunk32] = 1.0f / gb2;
+            if (p.comps > kCompsPlain) {
+                double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
+                                 __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
+                                 __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
+                o[10 * kChunk32] = __uint_as_float(p.n_sel ? selector_bits(p, x, ubd) : 0xffffffffu);
+            }
+            __syncthreads();
+            float* dst = p.slab32 + (tile * p.ring + slot0) * (p.comps * kTileP);
+            const int rec = p.comps * kChunk32;          // one particle's record
+            if (q * kChunk32 >= b.m0 && q * kChunk32 + kChunk32 - 1 <= b.m1) {
+                for (int v = tid; v < rec * kTileP / 4; v += 256) {
+                    const int r = v / (rec / 4), w = v - r * (rec / 4);
+                    reinterpret_cast<float4*>(dst)[v] =
+                        *reinterpret_cast<const float4*>(outs + r * ostride + 4 * w);
+                }
+            } else if (valid) {                          // the chunk's samples of this launch only
+                for (int c = 0; c < p.comps; ++c)
+                    dst[pp * rec + c * kChunk32 + sm] = outs[pp * ostride + c * kChunk32 + sm];
+            }
+        }
+        if (q == b.c1 && tid < 3 * kTileP && i >= 0) {
+            // the launch's last call is the state carried on (staged when other blocks
+            // of the launch may still be reading the state arrays)
+            const int c = tid >> 3, r = (int)(b.s1 - q * kChunk32);
+            const double nn = (double)(cnt[c][pp] - (any ? moved[c][pp] : 0));
+            const int64_t k = i - p.first;
+            double* sx = p.n_seg > 1 ? p.state_out + c * npart + k : p.x_prev + c * p.ncols + col;
+            double* sr = p.n_seg > 1 ? p.state_out + (3 + c) * npart + k : p.r_prev + c * p.ncols + col;
+            double* su = p.n_seg > 1 ? p.state_out + (6 + c) * npart + k : p.u_prev + c * p.ncols + col;
+            *sx = xs[r][c][pp];
+            *sr = nn;
+            *su = us[r][c][pp];
+        }
+        __syncthreads();
+        if (any && tid < 3 * kTileP) cnt[tid >> 3][pp] -= moved[tid >> 3][pp];
+    }
+    if (bad) atomicOr(p.err_word, kErrNaN);
+}
+
 IngestKernels ingest_kernel_ptr()
 {
     return {reinterpret_cast<const void*>(&ingest_kernel<false>),
             reinterpret_cast<const void*>(&ingest_kernel<true>)};
+}
+
+// A batch of calls through ingest_tile_kernel.
+static cudaError_t launch_batch(IngestParams q, int64_t cnt, cudaStream_t st)
+{
+    const BatchRange b = batch_range(q);
+    const int64_t chunks = b.c1 - b.c0 + 1;
+    // tiles of the launch's particles: all columns, or the range's (whole tiles of one
+    // species)
+    q.tile0 = 0;
+    q.n_tiles = (int32_t)(q.ncols / kTileP);
+    if (q.count || q.first) {
+        int sp = 0;
+        while (sp + 1 < q.n_species && q.first >= q.in_off[sp + 1]) ++sp;
+        const int64_t col = q.col_off[sp] + (q.first - q.in_off[sp]);
+        q.tile0 = col / kTileP;
+        q.n_tiles = (int32_t)((col + cnt - 1) / kTileP - q.tile0 + 1);
+    }
+    // Time segments (whole chunks) until the launch has about 8 blocks for every SM; from
+    // 608 tiles (4 blocks per SM) on the tiles alone do, and the extra pass over x for
+    // the image counts costs more than the shorter blocks give.
+    q.n_seg = 1;
+    q.seg_len = (int32_t)chunks;
+    if (q.n_tiles < kSegMaxTiles && q.state_out && (q.wind || !(q.box_L > 0.0))) {
+        const int64_t want = std::min<int64_t>(std::min<int64_t>(chunks, 1216 / q.n_tiles + 1), 250);
+        q.seg_len = (int32_t)((chunks + want - 1) / want);
+        q.n_seg = (int32_t)((chunks + q.seg_len - 1) / q.seg_len);
+    }
+    if (q.n_seg > 1 && q.box_L > 0.0) {
+        const int64_t nw = cnt * (q.n_seg - 1);
+        tile_wind_kernel<<<(unsigned)((nw + 127) / 128), 128, 0, st>>>(q);
+    }
+    const unsigned blocks = (unsigned)((int64_t)q.n_tiles * q.n_seg);
+    const size_t smem = q.slab32 ? (size_t)kTileP * (q.comps * kChunk32 + 4) * sizeof(float)
+                                 : (size_t)kChunk32 * 3 * kTileP * sizeof(int);
+    if (!q.slab32)
+        ingest_tile_kernel<2><<<blocks, 256, smem, st>>>(q);
+    else if (q.comps >= kCompsPrec)
+        ingest_tile_kernel<1><<<blocks, 256, smem, st>>>(q);
+    else
+        ingest_tile_kernel<0><<<blocks, 256, smem, st>>>(q);
+    if (q.n_seg > 1) store_state<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(q);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st)
@@ -422,10 +781,12 @@ cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st)
     if (cnt <= 0 || p.n_steps == 0) return cudaSuccess;
     IngestParams q = p;
     q.n_seg = 1;
+    // batches of calls; a few calls (below a quarter of a chunk) keep one thread per
+    // particle, and the sub-cycled samples their own loop
+    if (p.nsub <= 1 && p.n_steps >= 8) return launch_batch(q, cnt, st);
     // time segments only when the particles alone leave the GPU idle: with
     // 32,768 or more one thread per particle already keeps the FP64 pipes of
     // all SMs busy, and the segments' extra pass only adds work (measured)
-    constexpr int64_t kSegMaxParticles = 32768;
     if (p.wind && p.state_out && p.seg_len > 0 && cnt < kSegMaxParticles) {
         // boundaries at calls 1 + j seg_len strictly inside (step0, step0 + n_steps)
         // at most kMaxSeg segments (each thread sums the earlier segments' counts):

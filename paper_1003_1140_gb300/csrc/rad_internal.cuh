@@ -13,19 +13,23 @@ namespace rad {
 // ---------------------------------------------------------------------------
 // trajectory ring layout
 // ---------------------------------------------------------------------------
-// Both rings are tile-major: element (tile, slot, c, p) of particle column
-// col = 8 tile + p sits at ((tile * ring + slot) * comps + c) * 8 + p, so the
-// chunk of consecutive slots the kernels stage is one contiguous block.
+// Both rings are tile-major: particle column col is particle p = col % 8 of tile
+// col / 8.  FP64: element (tile, slot, c, p) sits at
+// ((tile * ring + slot) * comps + c) * 8 + p.  FP32: within each chunk of 32 slots
+// the samples are innermost, ((chunk * 8 + p) * comps + c) * 32 + slot % 32 with
+// chunk = (tile * ring + slot) / 32, so that a warp reads one particle's chunk
+// (contiguous, 1280 B) with lane = sample.  Either way the chunk of consecutive
+// slots the kernels stage is one contiguous block.
 // comps is 10, or 11 when sample selectors are defined (the flags word); the
 // precise-phase FP32 path adds dr's lo part as components 11-13 (comps 14).
-// FP32 split path: slab[tile][slot][c][p] float, c = 0..9 (10) =
+// FP32 split path: slab[tile][chunk][p][c][slot % 32] float, c = 0..9 (10) =
 //   dr (3)   : r_m - r_a, the offset from the block's FP64 anchor position
 //   beta (3) : beta_m
 //   bdot (3) : betadot_m (differenced in FP64 before the rounding)
 //   g (1)    : 1/gamma_m^2 = 1/(1 + ubar^2)
 //   flags (1): selector bits of the sample (bit i: inside selector i), stored as
 //              the float with those bits (FP32 ring) or as an exact double (FP64)
-// anc32[tile][blk][c][p] float, c = 0..5: r_a as hi (3) + lo (3) FP32 pairs at
+// anc32[tile][blk][p][c] float, c = 0..5: r_a as hi (3) + lo (3) FP32 pairs at
 //   the anchor samples a = K * blk (ring of ring/K blocks, tile-major like the
 //   samples, so a chunk's anchors are one contiguous block too).
 // FP64 path: slab64[tile][slot][c][p] double with c = r (3, absolute unwrapped),
@@ -39,6 +43,7 @@ constexpr int kChunk64 = 16;   // samples per TMA chunk, FP64 ring
 constexpr int kComputeWarps = 8;
 constexpr int kBlockThreads = (kComputeWarps + 1) * 32;  // + one TMA producer warp
 constexpr int kMaxSpecies = 32;
+constexpr int kFreqPad = 256;  // each grid's frequencies are padded with zeros to whole tiles
 
 // error word bits
 constexpr int kErrTimeout = 1;
@@ -61,7 +66,7 @@ struct WorkItem {
 // Per-window constants the accumulation kernels read.
 struct WinDev {
     int64_t s0, s1;      // sample range
-    int32_t grid_off;    // offset of the frequency grid in the frequency arrays
+    int32_t grid_off;    // offset of the frequency grid in the (padded) frequency arrays
     int32_t grid_len;    // frequencies in the grid
     int64_t out_off;     // offset of the window's [dirs][len] block in the accumulators
     int32_t sel;         // selector bit the samples must have, or -1 (all samples)
@@ -256,8 +261,10 @@ struct IngestParams {
     // anchor-aligned samples); wind [n_seg - 1][3][count] receives each
     // segment's change of the image count.  n_seg <= 1: one thread per particle.
     int64_t seg_first;
-    int32_t seg_len;
+    int32_t seg_len;        // calls (batched launches: 32-sample chunks) per segment
     int32_t n_seg;
+    int64_t tile0;          // batched launches: first tile and number of tiles
+    int32_t n_tiles;
     int32_t* wind;
     double* state_out;      // [9][count]: the last segment's carry-over state,
                             // stored to x_prev/r_prev/u_prev after the launch
@@ -302,6 +309,10 @@ struct Accum64Params {
     int32_t fault_stall;      // as in Accum32Params
 };
 
+// launch_ingest splits a launch in time below these sizes: 8-particle tiles (batches of
+// calls), particles (sub-cycled samples).
+constexpr int kSegMaxTiles = 608;
+constexpr int64_t kSegMaxParticles = 32768;
 cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st);
 // The two builds of the ingest kernel (common ring, precise-phase ring); a
 // kernel function pointer compares equal to the set when it is either build.
@@ -327,7 +338,11 @@ struct Accum32Config {
     bool band = false;   // items with anchor blocks of K << kmul (8 SFU frequencies per thread)
     int pm = 0;          // precise offset phase (8 SFU frequencies, K 32): 0 none, 1 every
                          // item, 2 the items whose WorkItem.prec is set
+    bool mom = false;    // block-moment kernel (the automatic choice): 8 frequencies per
+                         // thread, K 32
 };
+bool accum32_moment(const Accum32Params* p, const Accum32Config& cfg, int grid,
+                    cudaStream_t st, cudaError_t* err, int* nb);
 bool accum32_ft8_sfu(const Accum32Params* p, const Accum32Config& cfg, int grid,
                      cudaStream_t st, cudaError_t* err, int* nb);
 bool accum32_band(const Accum32Params* p, const Accum32Config& cfg, int grid,

@@ -96,9 +96,9 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     constexpr int K = 32;
     const int64_t S = n_calls - 1;                       // samples: window [0, S)
     const int64_t ncols = (N + kTileP - 1) / kTileP * kTileP;
-    const int64_t ring = (S + 31) / 32 * 32 + 64;
+    const int64_t ring = (S + 31) / 32 * 32;             // the one window, written once
     const int64_t nblk = ring / K;
-    const Accum32Config cfg{8, 0, K, coh, 2};
+    const Accum32Config cfg{8, 0, K, coh, 2, false, 0, true};   // the block-moment kernel
     const int ftl = 32 * cfg.ft;
     const int nft = (F + ftl - 1) / ftl;
     const int64_t ntiles = ncols / kTileP;
@@ -125,7 +125,8 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     const size_t o_state = cv.take<double>((size_t)9 * ncols);
     const size_t o_acc = cv.take<double>((size_t)D * F * (coh ? 4 : 1));
     const size_t o_dirs = cv.take<float>((size_t)D * 12);
-    const size_t o_om = cv.take<float>((size_t)3 * F);
+    const size_t Fp = ((size_t)F + kFreqPad - 1) / kFreqPad * kFreqPad;
+    const size_t o_om = cv.take<float>(3 * Fp);
     const size_t o_win = cv.take<WinDev>(1);
     const size_t o_sp = cv.take<SpeciesDev>(1);
     const size_t o_items = cv.take<WorkItem>((size_t)n_items);
@@ -168,8 +169,8 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
         if (!std::isfinite(freqs[k])) return RAD_EINVAL;
         const double nu = freqs[k] / 6.283185307179586476925286766559;
         ho[k] = (float)freqs[k];
-        ho[F + k] = (float)nu;
-        ho[2 * F + k] = (float)(nu - (double)(float)nu);
+        ho[Fp + k] = (float)nu;
+        ho[2 * Fp + k] = (float)(nu - (double)(float)nu);
     }
     WinDev* hw = reinterpret_cast<WinDev*>(host.data() + (o_win - t0));
     hw->s0 = 0;
@@ -237,8 +238,8 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     ap.species = reinterpret_cast<const SpeciesDev*>(B + o_sp);
     ap.dirs32 = reinterpret_cast<const float*>(B + o_dirs);
     ap.omega = reinterpret_cast<const float*>(B + o_om);
-    ap.nu_hi = ap.omega + F;
-    ap.nu_lo = ap.omega + 2 * F;
+    ap.nu_hi = ap.omega + Fp;
+    ap.nu_lo = ap.omega + 2 * Fp;
     ap.slab32 = ip.slab32;
     ap.anc32 = ip.anc32;
     ap.ring = ring;
