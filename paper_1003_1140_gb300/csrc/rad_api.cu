@@ -923,9 +923,11 @@ static int seg_scratch(rad_ctx* c, int64_t count, int64_t n_steps, IngestParams&
 }
 
 // Ingest n steps from device arrays x, u ([n][3][n_in]) starting at step0.
-static int ingest_device(rad_ctx* c, int64_t step0, int64_t n, const double* x, const double* u)
+static int ingest_device(rad_ctx* c, int64_t step0, int64_t n, const double* x, const double* u,
+                         int64_t ld = 0)
 {
     IngestParams p = ingest_params(c);
+    p.ld = ld;                             // 0: the particle axis is n_in long
     int64_t s = step0;
     const int64_t end = step0 + n;
     while (s < end) {
@@ -935,8 +937,8 @@ static int ingest_device(rad_ctx* c, int64_t step0, int64_t n, const double* x, 
             auto itv = c->event_at.lower_bound(s);
             if (itv != c->event_at.end() && itv->first < end) stop = itv->first + 1;
         }
-        p.x = x + (s - step0) * 3 * c->n_in;
-        p.u = u + (s - step0) * 3 * c->n_in;
+        p.x = x + (s - step0) * 3 * (ld ? ld : c->n_in);
+        p.u = u + (s - step0) * 3 * (ld ? ld : c->n_in);
         p.step0 = s;
         p.n_steps = (int32_t)(stop - s);
         int rs = seg_scratch(c, c->n_in, stop - s, p);
@@ -1230,9 +1232,10 @@ static int graph_for(rad_ctx* c, int kind, const IngestParams& ip, StepGraph** o
 }
 
 // One step through its graph: patch the ingest node's parameters, replay.
-static int step_via_graph(rad_ctx* c, int64_t step, const double* x, const double* u)
+static int step_via_graph(rad_ctx* c, int64_t step, const double* x, const double* u, int64_t ld)
 {
     IngestParams p = ingest_params(c);
+    p.ld = ld;
     p.x = x;
     p.u = u;
     p.n_steps = 1;
@@ -1293,10 +1296,86 @@ static int complete_windows(rad_ctx* c, F copy)
     return RAD_OK;
 }
 
+// The hand-over of n steps; ld: particle stride of device inputs (0: contiguous states).
+static int accumulate_impl(rad_ctx* c, int64_t step0, int64_t n, const double* x, const double* u,
+                           int64_t ld)
+{
+    if (!c) return RAD_EINVAL;
+    if (n < 0 || (n > 0 && (!x || !u))) return fail(c, RAD_EINVAL, "bad step count or null input");
+    if (step0 != c->next_step)
+        return fail(c, RAD_ESTEP, "step %lld given, %lld expected", (long long)step0,
+                    (long long)c->next_step);
+    if (n == 0) return RAD_OK;
+    if (c->fault.drop_step == step0) {   // test hook: this hand-over is lost once
+        c->fault.drop_step = -1;
+        return RAD_OK;
+    }
+    int rc = freeze(c);
+    if (rc) return rc;
+    CU(cudaSetDevice(c->device));
+    const bool dx = is_device_ptr(x), du = is_device_ptr(u);
+    if (dx && du && n == 1 && c->opt.use_graph && !c->graph_off &&
+        c->precision == RAD_FP32_SPLIT) {
+        rc = step_via_graph(c, step0, x, u, ld);
+        if (rc == kGraphUnavailable) {
+            c->graph_off = true;   // direct launches from now on
+            rc = ingest_device(c, step0, n, x, u, ld);
+        }
+        if (rc) return rc;
+    } else if (dx && du) {
+        rc = ingest_device(c, step0, n, x, u, ld);
+        if (rc) return rc;
+    } else if (!dx && !du && !c->opt.defer && n >= 64 && c->n_in >= 64 * kTileP * kHostBlocks) {
+        rc = ingest_host_blocked(c, step0, n, x, u);
+        if (rc) return rc;
+    } else {
+        // host inputs: double-buffered staging on a copy stream
+        const int64_t per = 3 * c->n_in;
+        int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n, 64));
+        if (c->stage_steps < chunk) {
+            for (int b = 0; b < 2; ++b) {
+                if (c->stage[b]) {
+                    CU(cudaStreamSynchronize(c->stream));
+                    CU(cudaFree(c->stage[b]));
+                    c->stage[b] = nullptr;
+                }
+                CU(cudaMalloc(&c->stage[b], (size_t)std::max<int64_t>(1, 2 * chunk * per) * sizeof(double)));
+            }
+            c->stage_steps = chunk;
+        }
+        for (int64_t s = 0; s < n; s += chunk) {
+            const int64_t m = std::min(chunk, n - s);
+            const int b = c->stage_next;
+            c->stage_next ^= 1;
+            double* sx = c->stage[b];
+            double* su = c->stage[b] + c->stage_steps * per;
+            CU(cudaStreamWaitEvent(c->copy_stream, c->used_done[b], 0));
+            const size_t bytes = (size_t)m * per * sizeof(double);
+            if (dx) CU(cudaMemcpyAsync(sx, x + s * per, bytes, cudaMemcpyDeviceToDevice, c->copy_stream));
+            else CU(cudaMemcpyAsync(sx, x + s * per, bytes, cudaMemcpyHostToDevice, c->copy_stream));
+            if (du) CU(cudaMemcpyAsync(su, u + s * per, bytes, cudaMemcpyDeviceToDevice, c->copy_stream));
+            else CU(cudaMemcpyAsync(su, u + s * per, bytes, cudaMemcpyHostToDevice, c->copy_stream));
+            CU(cudaEventRecord(c->copy_done[b], c->copy_stream));
+            CU(cudaStreamWaitEvent(c->stream, c->copy_done[b], 0));
+            rc = ingest_device(c, step0 + s, m, sx, su);
+            if (rc) return rc;
+            CU(cudaEventRecord(c->used_done[b], c->stream));
+        }
+        // the caller may reuse its host buffers once this returns
+        CU(cudaStreamSynchronize(c->copy_stream));
+    }
+    c->next_step = step0 + n;
+    return RAD_OK;
+}
+
 namespace rad {
 cudaStream_t ctx_stream(const rad_ctx* c) { return c ? c->stream : nullptr; }
 int64_t ctx_particles(const rad_ctx* c) { return c ? c->n_in : -1; }
 int64_t ctx_next_step(const rad_ctx* c) { return c ? c->next_step : -1; }
+int ctx_accumulate_strided(rad_ctx* c, int64_t step, const double* x, const double* u, int64_t ld)
+{
+    return accumulate_impl(c, step, 1, x, u, ld);
+}
 }  // namespace rad
 
 extern "C" {
@@ -1606,72 +1685,7 @@ int rad_get_options(const rad_ctx* c, rad_options* o)
 
 int rad_accumulate_steps(rad_ctx* c, int64_t step0, int64_t n, const double* x, const double* u)
 {
-    if (!c) return RAD_EINVAL;
-    if (n < 0 || (n > 0 && (!x || !u))) return fail(c, RAD_EINVAL, "bad step count or null input");
-    if (step0 != c->next_step)
-        return fail(c, RAD_ESTEP, "step %lld given, %lld expected", (long long)step0,
-                    (long long)c->next_step);
-    if (n == 0) return RAD_OK;
-    if (c->fault.drop_step == step0) {   // test hook: this hand-over is lost once
-        c->fault.drop_step = -1;
-        return RAD_OK;
-    }
-    int rc = freeze(c);
-    if (rc) return rc;
-    CU(cudaSetDevice(c->device));
-    const bool dx = is_device_ptr(x), du = is_device_ptr(u);
-    if (dx && du && n == 1 && c->opt.use_graph && !c->graph_off &&
-        c->precision == RAD_FP32_SPLIT) {
-        rc = step_via_graph(c, step0, x, u);
-        if (rc == kGraphUnavailable) {
-            c->graph_off = true;   // direct launches from now on
-            rc = ingest_device(c, step0, n, x, u);
-        }
-        if (rc) return rc;
-    } else if (dx && du) {
-        rc = ingest_device(c, step0, n, x, u);
-        if (rc) return rc;
-    } else if (!dx && !du && !c->opt.defer && n >= 64 && c->n_in >= 64 * kTileP * kHostBlocks) {
-        rc = ingest_host_blocked(c, step0, n, x, u);
-        if (rc) return rc;
-    } else {
-        // host inputs: double-buffered staging on a copy stream
-        const int64_t per = 3 * c->n_in;
-        int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n, 64));
-        if (c->stage_steps < chunk) {
-            for (int b = 0; b < 2; ++b) {
-                if (c->stage[b]) {
-                    CU(cudaStreamSynchronize(c->stream));
-                    CU(cudaFree(c->stage[b]));
-                    c->stage[b] = nullptr;
-                }
-                CU(cudaMalloc(&c->stage[b], (size_t)std::max<int64_t>(1, 2 * chunk * per) * sizeof(double)));
-            }
-            c->stage_steps = chunk;
-        }
-        for (int64_t s = 0; s < n; s += chunk) {
-            const int64_t m = std::min(chunk, n - s);
-            const int b = c->stage_next;
-            c->stage_next ^= 1;
-            double* sx = c->stage[b];
-            double* su = c->stage[b] + c->stage_steps * per;
-            CU(cudaStreamWaitEvent(c->copy_stream, c->used_done[b], 0));
-            const size_t bytes = (size_t)m * per * sizeof(double);
-            if (dx) CU(cudaMemcpyAsync(sx, x + s * per, bytes, cudaMemcpyDeviceToDevice, c->copy_stream));
-            else CU(cudaMemcpyAsync(sx, x + s * per, bytes, cudaMemcpyHostToDevice, c->copy_stream));
-            if (du) CU(cudaMemcpyAsync(su, u + s * per, bytes, cudaMemcpyDeviceToDevice, c->copy_stream));
-            else CU(cudaMemcpyAsync(su, u + s * per, bytes, cudaMemcpyHostToDevice, c->copy_stream));
-            CU(cudaEventRecord(c->copy_done[b], c->copy_stream));
-            CU(cudaStreamWaitEvent(c->stream, c->copy_done[b], 0));
-            rc = ingest_device(c, step0 + s, m, sx, su);
-            if (rc) return rc;
-            CU(cudaEventRecord(c->used_done[b], c->stream));
-        }
-        // the caller may reuse its host buffers once this returns
-        CU(cudaStreamSynchronize(c->copy_stream));
-    }
-    c->next_step = step0 + n;
-    return RAD_OK;
+    return accumulate_impl(c, step0, n, x, u, 0);
 }
 
 int rad_accumulate(rad_ctx* c, int64_t step, const double* x, const double* u)

@@ -329,6 +329,9 @@ cudaStream_t ctx_stream(const rad_ctx* c);
 // Particles a radiation context takes per call, and the step it expects next.
 int64_t ctx_particles(const rad_ctx* c);
 int64_t ctx_next_step(const rad_ctx* c);
+// rad_accumulate of one step from device arrays whose components are ld particles apart
+// (component c of particle i at x[c ld + i]), in the context's stream order.
+int ctx_accumulate_strided(rad_ctx* c, int64_t step, const double* x, const double* u, int64_t ld);
 // FP32 kernel variant: frequencies per thread, of which np by the FMA-pipe
 // polynomial, anchor interval K, coherent sum, minimum resident blocks per SM.
 struct Accum32Config {
