@@ -339,11 +339,12 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
             }
         }
         while (next_unit) {
-            const int v = L < 0 ? atomicAdd(p.counter, 1) : C.ticket;
+            // (with few units none is asked for early: it would wait while other warps idle)
+            const int v = L < 0 || p.few ? atomicAdd(p.counter, 1) : C.ticket;
             C.ii = -1;
             const int ii = v / kTileP;
             if (ii >= p.n_items) break;
-            C.ticket = atomicAdd(p.counter, 1);
+            if (!p.few) C.ticket = atomicAdd(p.counter, 1);
             const WorkItem it = p.items[ii];
             const SpeciesDev sp = p.species[it.sp];
             C.pp = v % kTileP;

@@ -106,6 +106,7 @@ struct rad_ctx {
     int64_t out_len = 0;
     rad_options opt{};
     Accum32Config cfg{8, 0, 16, false, 2};
+    int ft64 = 8;                  // FP64 path: frequency slots per lane
     int K = 16;                    // anchor interval used by the ingest
     bool per_band_K = false;       // FP32 path: each frequency tile's anchor blocks are the
                                    // longest multiple K << m within the phase budget
@@ -136,6 +137,8 @@ struct rad_ctx {
     float* d_nuhi = nullptr;
     float* d_nulo = nullptr;
     double* d_om64 = nullptr;
+    double* d_nu64 = nullptr;      // FP64 path: omega / 2 pi, hi then lo parts
+    double2* d_cis = nullptr;      // FP64 path: points of the unit circle
     WinDev* d_wins = nullptr;
     SelectorDev* d_sel = nullptr;
     int n_sel = 0;
@@ -280,11 +283,9 @@ bool rad::accum32_dispatch(const Accum32Params* p, const Accum32Config& cfg, int
            accum32_ft16(p, cfg, grid, st, err, nb) || accum32_ft4(p, cfg, grid, st, err, nb);
 }
 
-static int chunk_len(const rad_ctx* c) { return c->precision == RAD_FP64 ? kChunk64 : kChunk32; }
-
 static int freq_tile(const rad_ctx* c)
 {
-    return c->precision == RAD_FP64 ? 32 * accum64_ft() : 32 * c->cfg.ft;
+    return 32 * (c->precision == RAD_FP64 ? c->ft64 : c->cfg.ft);
 }
 
 static std::vector<std::vector<int>> band_kmul(const rad_ctx* c, int ftl);
@@ -300,7 +301,7 @@ static void build_items(rad_ctx* c, Event& ev, int total_blocks,
     auto lo_of = [&](int s) { return ranges ? (*ranges)[s].first : 0; };
     auto hi_of = [&](int s) { return ranges ? (*ranges)[s].second : INT_MAX; };
     const int ftl = freq_tile(c);
-    const int ch = chunk_len(c);
+    const int ch = kChunk32;
     // total (tile x direction x ftile) units, to size the particle groups
     double units = 0;
     for (int w : ev.wins) {
@@ -356,7 +357,8 @@ static void build_items(rad_ctx* c, Event& ev, int total_blocks,
 
 static int blocks_per_sm(const rad_ctx* c)
 {
-    if (c->precision == RAD_FP64) return std::max(1, accum64_blocks_per_sm(c->mode == RAD_COHERENT));
+    if (c->precision == RAD_FP64)
+        return std::max(1, accum64_blocks_per_sm(c->ft64, c->mode == RAD_COHERENT));
     int nb = 0;
     cudaError_t e = cudaSuccess;
     if (!accum32_dispatch(nullptr, c->cfg, 0, nullptr, &e, &nb)) return 0;
@@ -764,6 +766,22 @@ static int freeze(rad_ctx* c)
             if (rc) return rc;
         }
     }
+    if (c->precision == RAD_FP64) {
+        // the tile width of the window with the most work
+        double most = -1.0;
+        for (size_t w = 0; w < c->wins.size(); ++w) {
+            const rad_window& W = c->wins[w];
+            int64_t np = 0;
+            for (int s = 0; s < c->n_species; ++s)
+                if ((W.species_mask >> s) & 1u) np += c->species[s].count;
+            const int64_t pd = np * (int64_t)c->win_dirs[w].size();
+            const double work = (double)pd * (double)(W.s1 - W.s0) * c->grid_len[W.freq_grid];
+            if (work > most) {
+                most = work;
+                c->ft64 = accum64_ft(pd, c->grid_len[W.freq_grid], c->sms);
+            }
+        }
+    }
     // events
     c->events.clear();
     c->event_at.clear();
@@ -799,6 +817,17 @@ static int freeze(rad_ctx* c)
     return RAD_OK;
 }
 
+// Grid of an event's launch; few as unit_grid's (0 for the kernels whose blocks take whole
+// items).
+static int event_grid(const rad_ctx* c, const Event& ev, int32_t* few)
+{
+    const int total_blocks = blocks_per_sm(c) * c->sms;
+    *few = 0;
+    if (c->precision == RAD_FP64 || c->cfg.mom)
+        return unit_grid((int64_t)ev.items.size(), total_blocks, few);
+    return (int)std::min<int64_t>((int64_t)ev.items.size(), total_blocks);
+}
+
 // The stall hook applies to one launch only.
 static int32_t take_stall(rad_ctx* c)
 {
@@ -810,8 +839,8 @@ static int32_t take_stall(rad_ctx* c)
 static int launch_event(rad_ctx* c, Event& ev)
 {
     if (ev.items.empty()) return RAD_OK;
-    const int total_blocks = blocks_per_sm(c) * c->sms;
-    const int grid = (int)std::min<int64_t>((int64_t)ev.items.size(), total_blocks);
+    int32_t few = 0;
+    const int grid = event_grid(c, ev, &few);
     cudaEvent_t e0 = next_event(c->acc_ev, c->acc_used, true);
     CU(cudaEventRecord(e0, c->stream));
     cudaError_t e;
@@ -821,8 +850,13 @@ static int launch_event(rad_ctx* c, Event& ev)
         p.n_items = (int32_t)ev.items.size();
         p.wins = c->d_wins;
         p.species = c->d_species;
+        p.counter = c->d_counter;
+        p.few = few;
         p.dirs64 = c->d_dirs64;
         p.omega = c->d_om64;
+        p.nu_hi = c->d_nu64;
+        p.nu_lo = c->d_nu64 + c->h_freqs.size();
+        p.cis = c->d_cis;
         p.slab64 = c->slab64;
         p.ring = c->ring;
         p.comps = c->comps;
@@ -830,9 +864,11 @@ static int launch_event(rad_ctx* c, Event& ev)
         p.acc = c->acc;
         p.err_word = c->d_err;
         p.fault_stall = take_stall(c);
-        e = launch_accum64(p, c->mode == RAD_COHERENT, grid, c->stream);
+        CU(cudaMemsetAsync(c->d_counter, 0, sizeof(int), c->stream));
+        e = launch_accum64(p, c->ft64, c->mode == RAD_COHERENT, grid, c->stream);
     } else {
         Accum32Params p{};
+        p.few = few;
         p.items = ev.d_items;
         p.n_items = (int32_t)ev.items.size();
         p.counter = c->d_counter;
@@ -1178,8 +1214,8 @@ static int graph_for(rad_ctx* c, int kind, const IngestParams& ip, StepGraph** o
         if (e == cudaSuccess && kind > 0) {
             Event& ev = c->events[kind - 1];
             if (!ev.items.empty()) {
-                const int grid = (int)std::min<int64_t>((int64_t)ev.items.size(), blocks_per_sm(c) * c->sms);
                 Accum32Params p{};
+                const int grid = event_grid(c, ev, &p.few);
                 p.items = ev.d_items;
                 p.n_items = (int32_t)ev.items.size();
                 p.counter = c->d_counter;
@@ -1546,6 +1582,35 @@ int rad_init(rad_ctx** out, const double* dirs, int32_t D, const double* freqs,
     CUB(cudaMemcpy(c->d_wins, wd.data(), n_win * sizeof(WinDev), cudaMemcpyHostToDevice));
     CUB(cudaMemcpy(c->d_species, sd.data(), n_species * sizeof(SpeciesDev), cudaMemcpyHostToDevice));
 
+    if (precision == RAD_FP64) {
+        // nu = omega / 2 pi as a double-double (2 pi = two_pi + two_pi_lo) and the table
+        const double two_pi_lo = 2.4492935982947064e-16;
+        std::vector<double> nu(2 * nf);
+        for (int64_t i = 0; i < nf; ++i) {
+            nu[i] = c->h_freqs[i] / two_pi;
+            const double r = std::fma(-nu[i], two_pi, c->h_freqs[i]);
+            nu[nf + i] = std::fma(-nu[i], two_pi_lo, r) / two_pi;
+        }
+        const int nt = accum64_table();
+        std::vector<double2> tab(nt);
+        for (int k = 0; k < nt; ++k) {
+            // by the first octant's values, so that opposite points are exact mirrors
+            const int oct = k * 8 / nt, r = k - oct * nt / 8, q = (oct & 1) ? nt / 8 - r : r;
+            const double a = two_pi * q / nt, cs = std::cos(a), sn = std::sin(a);
+            const double u = (oct & 1) ? sn : cs, v = (oct & 1) ? cs : sn;
+            switch (oct >> 1) {
+                case 0: tab[k] = {u, v}; break;
+                case 1: tab[k] = {-v, u}; break;
+                case 2: tab[k] = {-u, -v}; break;
+                default: tab[k] = {v, -u}; break;
+            }
+        }
+        CUB(cudaMalloc(&c->d_nu64, nu.size() * sizeof(double)));
+        CUB(cudaMalloc(&c->d_cis, nt * sizeof(double2)));
+        CUB(cudaMemcpy(c->d_nu64, nu.data(), nu.size() * sizeof(double), cudaMemcpyHostToDevice));
+        CUB(cudaMemcpy(c->d_cis, tab.data(), nt * sizeof(double2), cudaMemcpyHostToDevice));
+    }
+
     // ring and state
     if (c->fault.alloc) return bail(RAD_ENOMEM);
     const int64_t nc = c->ncols;
@@ -1826,7 +1891,7 @@ void rad_destroy(rad_ctx* c)
         for (auto& ev : row) cudaFree(ev.d_items);
     void* bufs[] = {c->slab32, c->slab64, c->anc32, c->x_prev, c->r_prev, c->u_prev,
                     c->d_dirs32, c->d_dirs64, c->d_om32, c->d_nuhi, c->d_nulo,
-                    c->d_om64, c->d_wins, c->d_sel, c->d_species, c->acc, c->d_out, c->d_err, c->d_counter,
+                    c->d_om64, c->d_nu64, c->d_cis, c->d_wins, c->d_sel, c->d_species, c->acc, c->d_out, c->d_err, c->d_counter,
                     c->stage[0], c->stage[1], c->bstage[0], c->bstage[1], c->seg_buf};
     for (void* b : bufs)
         if (b) cudaFree(b);

@@ -112,11 +112,20 @@ __device__ uint32_t selector_bits(const IngestParams& p, const double x[3], cons
     return bits;
 }
 
-// Component 0 of a sample in the FP32 ring (components are kChunk32 apart).
-__device__ __forceinline__ float* slab32_at(const IngestParams& p, int64_t tile, int64_t slot, int64_t pp)
+// Component 0 of a sample in either ring (components are kChunk32 apart).
+template <class T>
+__device__ __forceinline__ T* slab_at(T* slab, const IngestParams& p, int64_t tile, int64_t slot,
+                                      int64_t pp)
 {
-    return p.slab32 + (((tile * p.ring + slot) / kChunk32 * kTileP + pp) * p.comps) * kChunk32 +
+    return slab + (((tile * p.ring + slot) / kChunk32 * kTileP + pp) * p.comps) * kChunk32 +
            slot % kChunk32;
+}
+
+// 1 / gamma of a momentum, FP64.  Written with explicit fused operations: both ingest
+// kernels have to give the same bits whatever surrounds the call.
+__device__ __forceinline__ double inv_gamma(double a, double b, double c)
+{
+    return rsqrt(fma(a, a, fma(b, b, fma(c, c, 1.0))));
 }
 
 // 64-thread blocks (launch_ingest), at least 8 resident per SM: the FP64-bound
@@ -276,7 +285,7 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                         }
                         have_anchor = true;
                     }
-                    float* o = slab32_at(p, tile, sl, pp);
+                    float* o = slab_at(p.slab32, p, tile, sl, pp);
                     for (int c = 0; c < 3; ++c) {
                         const double d = rk[c] - ra[c];
                         const float dh = (float)d;
@@ -288,14 +297,14 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                     o[9 * kChunk32] = (float)(1.0 / gk2);
                     if (p.comps > kCompsPlain) o[10 * kChunk32] = __uint_as_float(flags);
                 } else {
-                    double* o = p.slab64 + (tile * p.ring + sl) * (p.comps * kTileP) + pp;
+                    double* o = slab_at(p.slab64, p, tile, sl, pp);
                     for (int c = 0; c < 3; ++c) {
-                        o[c * kTileP] = rk[c];
-                        o[(3 + c) * kTileP] = bk[c];
-                        o[(6 + c) * kTileP] = bd[c];
+                        o[c * kChunk32] = rk[c];
+                        o[(3 + c) * kChunk32] = bk[c];
+                        o[(6 + c) * kChunk32] = bd[c];
                     }
-                    o[9 * kTileP] = 1.0 / gk2;
-                    if (p.comps > kCompsPlain) o[10 * kTileP] = (double)flags;
+                    o[9 * kChunk32] = 1.0 / gk2;
+                    if (p.comps > kCompsPlain) o[10 * kChunk32] = (double)flags;
                 }
             }
         } else if (p.slab32) {
@@ -337,7 +346,7 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             const float igq = 1.0f / gq;
             const float corr = dus / (gq * gm * (gq + gm));
             const float idt = (float)(1.0 / p.dt);
-            float* o = slab32_at(p, tile, slot, pp);
+            float* o = slab_at(p.slab32, p, tile, slot, pp);
             for (int c = 0; c < 3; ++c) {
                 const double d = rp[c] - ra[c];
                 const float dh = (float)d;
@@ -361,24 +370,21 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
         } else {
             double ub[3];
             for (int c = 0; c < 3; ++c) ub[c] = 0.5 * (up[c] + un[c]);
-            const double gm = sqrt(1.0 + (up[0] * up[0] + up[1] * up[1] + up[2] * up[2]));
-            const double gp = sqrt(1.0 + (un[0] * un[0] + un[1] * un[1] + un[2] * un[2]));
-            const double gb2 = 1.0 + (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
-            const double gb = sqrt(gb2);
-            double* o = p.slab64 + (tile * p.ring + slot) * (p.comps * kTileP) + pp;
-            o[0 * kTileP] = rp[0];
-            o[1 * kTileP] = rp[1];
-            o[2 * kTileP] = rp[2];
+            const double igm = inv_gamma(up[0], up[1], up[2]), igp = inv_gamma(un[0], un[1], un[2]);
+            const double igb = inv_gamma(ub[0], ub[1], ub[2]), idt64 = 1.0 / p.dt;
+            double* o = slab_at(p.slab64, p, tile, slot, pp);
             for (int c = 0; c < 3; ++c) {
-                o[(3 + c) * kTileP] = ub[c] / gb;
-                o[(6 + c) * kTileP] = (un[c] / gp - up[c] / gm) / p.dt;
+                o[c * kChunk32] = rp[c];
+                o[(3 + c) * kChunk32] = ub[c] * igb;
+                o[(6 + c) * kChunk32] =
+                    __dmul_rn(__dsub_rn(__dmul_rn(un[c], igp), __dmul_rn(up[c], igm)), idt64);
             }
-            o[9 * kTileP] = 1.0 / gb2;
+            o[9 * kChunk32] = igb * igb;
             if (p.comps > kCompsPlain) {
                 double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
                                  __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
                                  __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
-                o[10 * kTileP] = (double)(p.n_sel ? selector_bits(p, xp, ubd) : 0xffffffffu);
+                o[10 * kChunk32] = (double)(p.n_sel ? selector_bits(p, xp, ubd) : 0xffffffffu);
             }
         }
         for (int c = 0; c < 3; ++c) {
@@ -471,53 +477,59 @@ __device__ __forceinline__ int64_t tile_particle(const IngestParams& p, int64_t 
 }
 
 // Change of the image count over each segment but the last of a batched launch
-// (box_L > 0): one thread per particle and segment, eight calls' loads in flight.
+// (box_L > 0): a block per tile and segment, a thread per particle and chunk of 32
+// calls with eight calls' loads in flight (one thread per particle and whole segment
+// took 60 us for 1024 particles x 2000 calls, a chain of 28 load rounds).
 __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
 {
-    const int64_t cnt = p.count ? p.count : p.n_in - p.first;
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= cnt * (p.n_seg - 1)) return;
-    const int g = (int)(q / cnt);
-    const int64_t k = q - (int64_t)g * cnt, i = p.first + k;
-    const int64_t ld = p.ld ? p.ld : p.n_in, xi = i - p.xoff;
+    __shared__ int tot[3][kTileP];
+    const int tid = threadIdx.x, pp = tid & (kTileP - 1);
+    const int tile_l = (int)(blockIdx.x % p.n_tiles), g = (int)(blockIdx.x / p.n_tiles);
+    const int64_t col = (p.tile0 + tile_l) * kTileP + pp;
+    const int64_t i = tile_particle(p, col);
+    const int64_t npart = p.count ? p.count : p.n_in - p.first;
+    const int64_t ld = p.ld ? p.ld : p.n_in;
     const BatchRange b = batch_range(p);
-    // calls (sa, sb] of the segment's samples
-    const int64_t sa = g == 0 ? b.m0 : (b.c0 + (int64_t)g * p.seg_len) * kChunk32;
-    const int64_t sb = (b.c0 + (int64_t)(g + 1) * p.seg_len) * kChunk32;
     const float lim = 0.4999f * (float)p.box_L;
     const double half_L = 0.5 * p.box_L;
-    const double* x = p.x + xi;
-    double xp[3];
-    int32_t dn[3] = {0, 0, 0};
+    if (tid < 3 * kTileP) tot[tid >> 3][pp] = 0;
+    __syncthreads();
+    int dn[3] = {0, 0, 0};
+    if (i >= 0) {
+        const double* x = p.x + (i - p.xoff);
+        for (int q = tid >> 3; q < p.seg_len; q += 32) {
+            // calls (sa, sb] of chunk q of the segment
+            const int64_t c = b.c0 + (int64_t)g * p.seg_len + q;
+            const int64_t sa = max(b.m0, c * kChunk32), sb = (c + 1) * kChunk32;
+            double xp[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        if (sa >= p.step0) {
-            xp[c] = x[((sa - p.step0) * 3 + c) * ld];
-        } else {
-            int sp = 0;
-            while (sp + 1 < p.n_species && i >= p.in_off[sp + 1]) ++sp;
-            xp[c] = p.x_prev[c * p.ncols + p.col_off[sp] + (i - p.in_off[sp])];
-        }
-    }
-    constexpr int U = 8;
-    for (int64_t s = sa + 1; s <= sb; s += U) {
-        double xn[U][3];
+            for (int k = 0; k < 3; ++k)
+                xp[k] = sa >= p.step0 ? x[((sa - p.step0) * 3 + k) * ld] : p.x_prev[k * p.ncols + col];
+            constexpr int U = 8;
+            for (int64_t s = sa + 1; s <= sb; s += U) {
+                double xn[U][3];
 #pragma unroll
-        for (int j = 0; j < U; ++j)
+                for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-                xn[j][c] = x[((min(s + j, sb) - p.step0) * 3 + c) * ld];
+                    for (int k = 0; k < 3; ++k)
+                        xn[u][k] = x[((min(s + u, sb) - p.step0) * 3 + k) * ld];
 #pragma unroll
-        for (int j = 0; j < U; ++j)
+                for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                if (maybe_jump(xp[c], xn[j][c], lim))
-                    dn[c] -= (int32_t)image_jump(xn[j][c] - xp[c], p.box_L, half_L);
-                xp[c] = xn[j][c];
+                    for (int k = 0; k < 3; ++k) {
+                        if (maybe_jump(xp[k], xn[u][k], lim))
+                            dn[k] -= (int)image_jump(xn[u][k] - xp[k], p.box_L, half_L);
+                        xp[k] = xn[u][k];
+                    }
             }
-    }
+        }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) p.wind[((int64_t)g * 3 + c) * cnt + k] = dn[c];
+        for (int k = 0; k < 3; ++k)
+            if (dn[k]) atomicAdd(&tot[k][pp], dn[k]);
+    }
+    __syncthreads();
+    if (tid < 3 * kTileP && i >= 0)
+        p.wind[((int64_t)g * 3 + (tid >> 3)) * npart + (i - p.first)] = tot[tid >> 3][pp];
 }
 
 // One block: chunks [q0, q1) (32 samples each) of one 8-particle tile, thread = sample
@@ -528,16 +540,18 @@ __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
 // ran 27 FP64 instructions per sample and a serial chain over the calls: 192 us for
 // 1024 particles x 2000 calls).  The record of a chunk is staged in shared memory and
 // written as one contiguous block.  MODE 0: FP32 ring, 1: the precise-phase FP32 ring
-// (the offsets' lo part too), 2: FP64 ring (its 16-sample chunks have the same order of
-// slots; samples are written directly).
+// (the offsets' lo part too), 2: FP64 ring (samples written directly, four to a sector).
 template <int MODE>
 __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(const IngestParams p)
 {
     __shared__ double xs[kChunk32 + 1][3][kTileP], us[kChunk32 + 1][3][kTileP];
     __shared__ double ras[kChunk32 / 8][3][kTileP];
     __shared__ int cnt[3][kTileP], moved[3][kTileP];
-    extern __shared__ __align__(16) float outs[];       // [particle][comp][sample], padded
+    // FP32: [particle][comp][sample], padded; FP64: beta at the half steps.  Before that,
+    // the crossings of a chunk that has any.
+    extern __shared__ __align__(16) float outs[];
     int(*jc)[3][kTileP] = reinterpret_cast<int(*)[3][kTileP]>(outs);
+    double(*bh)[3][kTileP] = reinterpret_cast<double(*)[3][kTileP]>(outs);
     const int tid = threadIdx.x, sm = tid >> 3, pp = tid & (kTileP - 1);
     const int tile_l = (int)(blockIdx.x % p.n_tiles), g = (int)(blockIdx.x / p.n_tiles);
     const int64_t tile = p.tile0 + tile_l, col = tile * kTileP + pp;
@@ -549,7 +563,8 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
     const int64_t q1 = min(q0 + p.seg_len, b.c1 + 1);
     const bool box = p.box_L > 0.0;
     const float lim = 0.4999f * (float)p.box_L;
-    const float idt = (float)(1.0 / p.dt);
+    const double idt64 = 1.0 / p.dt;
+    const float idt = (float)idt64;
     const int ostride = p.comps * kChunk32 + 4;
     bool bad = false;
 
@@ -636,25 +651,32 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
         }
         if (any) __syncthreads();
         if (MODE == 2) {
+            // beta at the half steps, once per call (a sample uses two neighbouring ones):
+            // one reciprocal square root where the samples took three square roots and
+            // ten divisions between them (154 FP64 instructions each)
+            auto half = [&](int r) {
+                const double ig = inv_gamma(us[r][0][pp], us[r][1][pp], us[r][2][pp]);
+                for (int c = 0; c < 3; ++c) bh[r][c][pp] = __dmul_rn(us[r][c][pp], ig);
+            };
+            half(sm);
+            if (sm == 0) half(kChunk32);
+            __syncthreads();
             if (valid && i >= 0) {
                 double ub[3];
                 for (int c = 0; c < 3; ++c) ub[c] = 0.5 * (up[c] + un[c]);
-                const double gm = sqrt(1.0 + (up[0] * up[0] + up[1] * up[1] + up[2] * up[2]));
-                const double gp = sqrt(1.0 + (un[0] * un[0] + un[1] * un[1] + un[2] * un[2]));
-                const double gb2 = 1.0 + (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
-                const double gb = sqrt(gb2);
-                double* o = p.slab64 + (tile * p.ring + slot0 + sm) * (p.comps * kTileP) + pp;
+                const double igb = inv_gamma(ub[0], ub[1], ub[2]);
+                double* o = slab_at(p.slab64, p, tile, slot0 + sm, pp);
                 for (int c = 0; c < 3; ++c) {
-                    o[c * kTileP] = x[c] + p.box_L * (double)n[c];
-                    o[(3 + c) * kTileP] = ub[c] / gb;
-                    o[(6 + c) * kTileP] = (un[c] / gp - up[c] / gm) / p.dt;
+                    o[c * kChunk32] = n[c] ? __dadd_rn(x[c], __dmul_rn(p.box_L, (double)n[c])) : x[c];
+                    o[(3 + c) * kChunk32] = ub[c] * igb;
+                    o[(6 + c) * kChunk32] = __dmul_rn(__dsub_rn(bh[sm + 1][c][pp], bh[sm][c][pp]), idt64);
                 }
-                o[9 * kTileP] = 1.0 / gb2;
+                o[9 * kChunk32] = igb * igb;
                 if (p.comps > kCompsPlain) {
                     double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
                                      __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
                                      __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
-                    o[10 * kTileP] = (double)(p.n_sel ? selector_bits(p, x, ubd) : 0xffffffffu);
+                    o[10 * kChunk32] = (double)(p.n_sel ? selector_bits(p, x, ubd) : 0xffffffffu);
                 }
             }
         } else {
@@ -758,13 +780,11 @@ static cudaError_t launch_batch(IngestParams q, int64_t cnt, cudaStream_t st)
         q.seg_len = (int32_t)((chunks + want - 1) / want);
         q.n_seg = (int32_t)((chunks + q.seg_len - 1) / q.seg_len);
     }
-    if (q.n_seg > 1 && q.box_L > 0.0) {
-        const int64_t nw = cnt * (q.n_seg - 1);
-        tile_wind_kernel<<<(unsigned)((nw + 127) / 128), 128, 0, st>>>(q);
-    }
+    if (q.n_seg > 1 && q.box_L > 0.0)
+        tile_wind_kernel<<<(unsigned)((int64_t)q.n_tiles * (q.n_seg - 1)), 256, 0, st>>>(q);
     const unsigned blocks = (unsigned)((int64_t)q.n_tiles * q.n_seg);
     const size_t smem = q.slab32 ? (size_t)kTileP * (q.comps * kChunk32 + 4) * sizeof(float)
-                                 : (size_t)kChunk32 * 3 * kTileP * sizeof(int);
+                                 : (size_t)(kChunk32 + 1) * 3 * kTileP * sizeof(double);
     if (!q.slab32)
         ingest_tile_kernel<2><<<blocks, 256, smem, st>>>(q);
     else if (q.comps >= kCompsPrec)

@@ -14,12 +14,11 @@ namespace rad {
 // trajectory ring layout
 // ---------------------------------------------------------------------------
 // Both rings are tile-major: particle column col is particle p = col % 8 of tile
-// col / 8.  FP64: element (tile, slot, c, p) sits at
-// ((tile * ring + slot) * comps + c) * 8 + p.  FP32: within each chunk of 32 slots
-// the samples are innermost, ((chunk * 8 + p) * comps + c) * 32 + slot % 32 with
+// col / 8.  Within each chunk of 32 slots the samples are innermost: element
+// (tile, slot, c, p) sits at ((chunk * 8 + p) * comps + c) * 32 + slot % 32 with
 // chunk = (tile * ring + slot) / 32, so that a warp reads one particle's chunk
-// (contiguous, 1280 B) with lane = sample.  Either way the chunk of consecutive
-// slots the kernels stage is one contiguous block.
+// (contiguous, 1280 B in FP32) with lane = sample; the chunk of all eight particles is
+// one contiguous block too.
 // comps is 10, or 11 when sample selectors are defined (the flags word); the
 // precise-phase FP32 path adds dr's lo part as components 11-13 (comps 14).
 // FP32 split path: slab[tile][chunk][p][c][slot % 32] float, c = 0..9 (10) =
@@ -32,14 +31,13 @@ namespace rad {
 // anc32[tile][blk][p][c] float, c = 0..5: r_a as hi (3) + lo (3) FP32 pairs at
 //   the anchor samples a = K * blk (ring of ring/K blocks, tile-major like the
 //   samples, so a chunk's anchors are one contiguous block too).
-// FP64 path: slab64[tile][slot][c][p] double with c = r (3, absolute unwrapped),
+// FP64 path: slab64[tile][chunk][p][c][slot % 32] double with c = r (3, absolute unwrapped),
 // beta (3), bdot (3), g (1), flags (1).
 constexpr int kComps = 11;     // components at most (10 + the selector flags)
 constexpr int kCompsPlain = 10;   // without selectors
 constexpr int kCompsPrec = 14;    // precise-phase FP32 ring: + flags + the lo part of dr
 constexpr int kTileP = 8;      // particles per tile: one warp each
-constexpr int kChunk32 = 32;   // samples per TMA chunk, FP32 ring
-constexpr int kChunk64 = 16;   // samples per TMA chunk, FP64 ring
+constexpr int kChunk32 = 32;   // samples per chunk
 constexpr int kComputeWarps = 8;
 constexpr int kBlockThreads = (kComputeWarps + 1) * 32;  // + one TMA producer warp
 constexpr int kMaxSpecies = 32;
@@ -274,6 +272,7 @@ struct Accum32Params {
     const WorkItem* items;
     int32_t n_items;
     int* counter;             // dynamic item counter (zeroed before the launch)
+    int32_t few;              // block-moment kernel: unit_grid's few
     const WinDev* wins;
     const SpeciesDev* species;
     const float* dirs32;      // [D][12]: n, e1, e2, n - (float)n
@@ -298,8 +297,13 @@ struct Accum64Params {
     int32_t n_items;
     const WinDev* wins;
     const SpeciesDev* species;
+    int* counter;             // dynamic unit counter (zeroed before the launch)
+    int32_t few;              // unit_grid's few
     const double* dirs64;     // [D][9]: n, e1, e2
     const double* omega;      // [n_freq]
+    const double* nu_hi;      // [n_freq] omega / 2 pi, hi and lo part
+    const double* nu_lo;
+    const double2* cis;       // [accum64_table()] cos, sin of 2 pi j / table
     const double* slab64;     // tile-major FP64 ring
     int64_t ring;
     int32_t comps;            // ring components per sample (10, or 11 with selector flags)
@@ -361,8 +365,18 @@ bool accum32_ft4(const Accum32Params* p, const Accum32Config& cfg, int grid,
 // launch (p != nullptr) or occupancy query; false if the variant is not built
 bool accum32_dispatch(const Accum32Params* p, const Accum32Config& cfg, int grid,
                       cudaStream_t st, cudaError_t* err, int* nb);
-cudaError_t launch_accum64(const Accum64Params& p, bool coh, int grid, cudaStream_t st);
-int accum64_blocks_per_sm(bool coh);
-int accum64_ft();
+// FP64 kernel with ft frequency slots per lane (2, 4 or 8)
+cudaError_t launch_accum64(const Accum64Params& p, int ft, bool coh, int grid, cudaStream_t st);
+int accum64_blocks_per_sm(int ft, bool coh);
+// Grid of the kernels whose warps take units (an item's particles) on their own: the full
+// grid, so that all SMs get the same number of blocks.  few: under four units per warp,
+// each unit is taken only when a warp is free for it.
+inline int unit_grid(int64_t n_items, int total_blocks, int32_t* few)
+{
+    *few = n_items * kTileP < (int64_t)4 * 4 * total_blocks;
+    return total_blocks;
+}
+int accum64_ft(int64_t particle_dirs, int n_omega, int sms);
+int accum64_table();
 
 }  // namespace rad

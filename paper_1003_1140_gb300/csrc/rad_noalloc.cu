@@ -249,7 +249,7 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     ap.dt_lo = (float)(dt - (double)ap.dt_hi);
     ap.acc = reinterpret_cast<double*>(B + o_acc);
     ap.err_word = err_word;
-    const int grid = (int)std::min<int64_t>(n_items, total_blocks);
+    const int grid = unit_grid(n_items, total_blocks, &ap.few);
     if (!accum32_dispatch(&ap, cfg, grid, st, &e, nullptr)) return RAD_ECUDA;
     NA_CU(e);
 

@@ -59,6 +59,28 @@ def test_frequency_slots_and_orders(traj, nw, coherent):
     _close(got, ref, TOL)
 
 
+@pytest.mark.parametrize("ndir,nw", [(3, 33), (3, 130), (40, 300), (100, 70), (100, 300)])
+@pytest.mark.parametrize("coherent", [False, True])
+def test_fp64_tile_widths(traj, ndir, nw, coherent):
+    """The FP64 kernel's three tile widths (chosen by the number of units), frequencies from
+    moments to direct sums, shuffled and signed: within 1e-10 of the oracle."""
+    import paper_1003_1140_gb300 as R
+    w, X, U = traj
+    rng = np.random.default_rng(ndir + nw)
+    dirs = rng.normal(size=(ndir, 3))        # the library normalises, the oracle takes unit vectors
+    unit = dirs / np.linalg.norm(dirs, axis=1, keepdims=True)
+    a = trajgen.log_grid(0.002, 200.0, nw)
+    grids = [a, rng.permutation(a) * rng.choice([-1.0, 1.0], nw)]
+    wins = [(0, 230, 3, 0), (13, 77, 1, 1)]
+    sp = [(s[0], s[1]) for s in w.species]
+    ref = oracle.spectra(X, U, w.dt, unit, grids, wins, sp, coherent=coherent, box_L=3.0)
+    with R.Radiation(dirs, grids, w.dt, [s[:3] for s in w.species], wins, precision=R.RAD_FP64,
+                     mode=R.RAD_COHERENT if coherent else R.RAD_INCOHERENT, box_L=3.0) as r:
+        r.accumulate_steps(0, torch.as_tensor(X, device="cuda"), torch.as_tensor(U, device="cuda"))
+        got = r.finalize()
+    _close(got, ref, 1e-10)
+
+
 @pytest.mark.parametrize("cuts", [[0, 231], [0, 8, 17, 49, 81, 231], [0, 1, 33, 65, 66, 230, 231],
                                   [0, 32, 64, 128, 200, 231], [0, 7, 20, 31, 47, 160, 231]])
 @pytest.mark.parametrize("opts", ["fp64", None, {"variant": 1, "anchor_K": 8}, {"variant": 3}])
