@@ -73,7 +73,7 @@ int rad_mlp_set_transform(rad_mlp *m, const float *in_mu, const float *in_sd, co
 int rad_mlp_predict(rad_mlp *m, int32_t batch, const float *x, float *y);
 
 /* One Adam step from the stored gradients (bias-corrected; FP32 master weights,
- * BF16 copies of W and W^T refreshed).  Stream ordered; does not wait. */
+ * BF16 copy of W refreshed).  Stream ordered; does not wait. */
 int rad_mlp_adam(rad_mlp *m, float lr, float beta1, float beta2, float eps);
 
 /* One training step: rad_mlp_gradients followed by rad_mlp_adam in one call,
@@ -85,9 +85,9 @@ int rad_mlp_train_step(rad_mlp *m, int32_t batch, const float *x, const float *t
                        float beta1, float beta2, float eps, double *loss);
 
 /* The tensor-core GEMM on its own: C [M][N] (FP32, device) = op(A) op(B), BF16
- * device operands (16-byte aligned); a_kcontig != 0: A stored [M][K], else
- * [K][M]; b_kcontig != 0: B stored [N][K], else [K][N] (operands stored K-last are first
- * transposed into scratch).  M, N multiples of 128, K of 64.  Default stream;
+ * device operands (A [M][K], B [N][K] and C 16-byte aligned); a_kcontig != 0: A stored [M][K], else
+ * [K][M]; b_kcontig != 0: B stored [N][K], else [K][N] (read in place;
+ * one that is not 16-byte aligned is copied into scratch first).  M, N multiples of 128, K of 64.  Default stream;
  * returns once the work is enqueued.  Products with few 128 x 128 output tiles
  * and a long K are split over K.  Scratch comes from the default stream's
  * stream-ordered pool (RAD_MLP_ENOMEM when it cannot be had).  A, B or C
