@@ -248,14 +248,18 @@ __device__ __forceinline__ void eval_moments(const float4* M, f2 x, f2 nx, f2 th
     a2i = fma2(O2, c, a2i);
 }
 
-// Direct sum of samples [lo, hi) for the slot pairs A .. B - 1.
-template <int A, int B>
+// Direct sum of samples [lo, hi) for the slot pairs A .. B - 1.  With one or two pairs a
+// sample's chain (load, phase, sine, sums) is not hidden by the other pairs': several samples
+// at once (UNROLL) take the 64-frequency subset of 1024 particles from 1.51 to 1.38 ms; the
+// coherent kernel, short of registers, gets slower by it (9.05 to 9.5 ms) and does without.
+template <int A, int B, bool UNROLL>
 __device__ __forceinline__ void direct_sum(const float4* geo, int lo, int hi, const f2 (&om)[kPairs],
                                            const f2 (&th)[kPairs], f2 (&a1r)[kPairs],
                                            f2 (&a1i)[kPairs], f2 (&a2r)[kPairs], f2 (&a2i)[kPairs])
 {
+    constexpr int U = !UNROLL || B - A > 2 ? 1 : 4 / (B - A);
     float4 g = geo[lo];
-#pragma unroll 1
+#pragma unroll U
     for (int l = lo; l < hi; ++l) {
         const float4 gn = geo[l + 1];    // [32] is padding
         const f2 v1 = dup(g.x), v2 = dup(g.y), dp = dup(g.z);
@@ -639,13 +643,13 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
                 }
             }
             switch (da + 4 * (kPairs - db)) {
-                case 0: direct_sum<0, 4>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 1: direct_sum<1, 4>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 2: direct_sum<2, 4>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 3: direct_sum<3, 4>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 4: direct_sum<0, 3>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 8: direct_sum<0, 2>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 12: direct_sum<0, 1>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 0: direct_sum<0, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 1: direct_sum<1, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 2: direct_sum<2, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 3: direct_sum<3, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 4: direct_sum<0, 3, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 8: direct_sum<0, 2, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
+                case 12: direct_sum<0, 1, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
                 default: break;
             }
         }
