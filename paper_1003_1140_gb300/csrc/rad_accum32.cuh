@@ -419,8 +419,12 @@ __global__ void __launch_bounds__(kBlockThreads, MB) accum32_kernel(const Accum3
                 S.anc[buf][pp][B] = make_float2(hi, e - (hi - sh));
             }
             __syncwarp();
-            // geometry: round r handles particle r, lane = sample
-#pragma unroll 2
+            // geometry: round r handles particle r, lane = sample.  One round at a time (2048
+            // particles of the precision workload, 2 blocks per SM: SFU build 31.1 ms against
+            // 33.1 unrolled by two, MIX 33.9 against 35.1); the precise phase's longer chain
+            // wants two (45.3 against 47.5 ms).
+            constexpr int kRounds = PM ? 2 : 1;
+#pragma unroll kRounds
             for (int r = 0; r < kTileP; ++r) {
                 const int sm = lane, pp = r;
                 const float* tb = &S.tbuf[buf][0] + pp * pstride + sm;
