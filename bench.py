@@ -46,8 +46,8 @@ METRIC = "G particle·step·ω·n updates/s, FP32 split vs FP64 GPU at ≤1e-4 r
 # workload scaled to 4096 particles (same samples, directions and omegas), valid while
 # the code (comments aside) of the kernel and of its work-list builder is the code that
 # was captured; traffic scales with the particle count.
-TRAFFIC_CAPTURE = {"sources_sha256": "cadabcb64484e3e00e449b1f01f7142ba83ff5aac4b20d3cd0e4aa48eb6da180",
-                   "bytes_per_launch": 699.964416e6, "particles": 4096}
+TRAFFIC_CAPTURE = {"sources_sha256": "87c83b2a22f963484847d69087a3730ce3fd44a5ed1a7429273fc360c99d5269",
+                   "bytes_per_launch": 695.9e6, "particles": 4096}
 UNIT = "G updates/s"
 # phase budget (rad per update) of the accuracy side-run: the upper decade of the
 # precision workload's grid (dt 0.05, w <= 1000) takes anchor blocks of 8 samples
@@ -172,7 +172,9 @@ def traffic_sources_hash() -> str:
     the host library that builds its work list and launches it."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("paper_1003_1140_gb300/csrc/rad_accum32.cuh", "paper_1003_1140_gb300/csrc/rad_api.cu"):
+    for f in ("paper_1003_1140_gb300/csrc/rad_accum32.cuh",
+              "paper_1003_1140_gb300/csrc/rad_accum32_moment.cu",
+              "paper_1003_1140_gb300/csrc/rad_api.cu"):
         with open(os.path.join(ROOT, f), encoding="utf-8") as fh:
             h.update(code_only(fh.read()).encode())
     return h.hexdigest()

@@ -1,7 +1,12 @@
-"""Roofline of the FP32 split-phase accumulation kernel (an ALU-bound kernel).
+"""Roofline of the FP32 split-phase accumulation (ALU-bound), evaluated sample by sample.
 
-The work unit is an update per (particle, sample, direction, omega).  The
-algorithmic minimum per update is one FFMA for the phase theta = w dphi +
+The work unit is an update per (particle, sample, direction, omega).  The bounds are
+those of the direct sum, in which every update is evaluated on its own.  The automatic
+kernel takes the moments of whole blocks of samples where the phase allows it and does
+less work than that, so its rate may pass the special-function and issue bounds; the
+explicit variants stay below them.
+
+The direct sum's minimum per update is one FFMA for the phase theta = w dphi +
 Theta, six FFMA to add V e^{i theta} to the three complex components of the
 amplitude, and e^{i theta} itself: two special-function (MUFU) operations
 (sin, cos), or an FMA-pipe polynomial of P instructions.  Per-SM unit counts
@@ -18,7 +23,7 @@ of sm_103a:
   p = 17/26 and 8 / p = 208/17 = 12.24 updates / clock / SM.
 * SFU bound: every e^{i theta} on the MUFU pipe, 2 MUFU per update ->
   16 / 2 = 8 updates / clock / SM.
-* Issue model of this kernel's own instruction stream (reported beside the
+* Issue model of the direct kernels' own instruction stream (reported beside the
   others): 5 FFMA (V has two components on a basis normal to n, so the
   amplitude needs two complex accumulators: 4 FFMA, plus the phase), the
   argument-scale FMUL and 2 MUFU on the SFU path or a 17-instruction
@@ -37,7 +42,7 @@ ISSUE_PER_CLK = 128.0
 # algorithmic count
 ALG_FP32 = 7.0             # phase FFMA + 6 accumulate FFMA
 ALG_POLY = 10.0            # FMA-pipe sin/cos polynomial of the algorithmic bound
-# this kernel's instruction stream
+# the direct kernels' instruction stream
 COMMON_FP32 = 5.0          # phase FFMA + 4 accumulate FFMA
 SFU_PATH_ISSUE = 3.0       # argument-scale FMUL + MUFU.SIN + MUFU.COS
 POLY_FP32 = 17.0           # Cody-Waite half-turn reduction (4), y^2 (1), sin deg 9 (5),
@@ -66,7 +71,7 @@ def algorithmic_per_clk(fp32: float = ALG_FP32, poly: float = ALG_POLY):
 
 
 def combined_per_clk(poly_fp32: float = POLY_FP32):
-    """Best updates/clock/SM of this kernel's issue model over p, and that p."""
+    """Best updates/clock/SM of the direct kernels' issue model over p, and that p."""
     return _best(lambda p: max((COMMON_FP32 + SFU_PATH_ISSUE * p + poly_fp32 * (1.0 - p))
                                / ISSUE_PER_CLK, 2.0 * p / MUFU_PER_CLK))
 
@@ -88,6 +93,6 @@ def accum32_roofline(updates_per_launch: float, ms_per_launch: float, sms: int,
             "peak_sfu": peak_sfu, "frac_sfu": achieved / peak_sfu if peak_sfu else None,
             "peak_issue_model": peak_issue,
             "frac_issue_model": achieved / peak_issue if peak_issue else None,
-            "issue_model_kind": f"this kernel's stream: 5 FFMA + (FMUL + 2 MUFU | 17-op "
+            "issue_model_kind": f"the direct sum's stream: 5 FFMA + (FMUL + 2 MUFU | 17-op "
                                 f"polynomial), {comb:.2f} updates/clk/SM at p_sfu={p:.2f}",
             "ms_per_launch": ms_per_launch, "updates_per_launch": updates_per_launch}
