@@ -8,7 +8,7 @@
 //   M_p = sum_m V_m (dphi_m / h)^p,   |dphi_m| <= h,
 // with c_p the coefficients of polynomials for cos and sin on |w h| <= X0.
 // The M_p (real, two components of V) do not depend on the frequency: one warp
-// forms them once per chunk, lane = sample, and every frequency then costs P
+// forms them once per chunk, lane = sample, and every frequency then costs P = 12
 // multiply-adds per component and one rotation per chunk instead of 32 sines,
 // cosines and 128 multiply-adds.  Larger w h are halved by splitting the chunk
 // into two or four sub-blocks about their own centres; beyond that (or for
@@ -93,16 +93,17 @@ constexpr int kMaxP = 12;    // moments per sub-block
 
 // Polynomials cos t = sum_j C_j (-t^2)^j, sin t = t sum_j S_j (-t^2)^j, leading
 // coefficients exactly 1, the rest minimax fits with successively rounded
-// coefficients (fit_sincos.py, fit_moment): P = 8 terms to 6.1e-8 on |t| <= 0.85,
-// P = 12 terms to 6.1e-8 on |t| <= 2.5 -- an eighth of the special-function
-// unit's own error, so the moments never lose accuracy against the direct sum.
-constexpr float kX8 = 0.85f, kX12 = 2.5f;
-__device__ const float g_moment_coef[2][kMaxP] = {
-    {1.0f, 1.0f, 4.999983013e-01f, 1.666664034e-01f, 4.165240005e-02f, 8.331445977e-03f,
-     1.354771084e-03f, 1.943349489e-04f, 0.0f, 0.0f, 0.0f, 0.0f},
-    {1.0f, 1.0f, 4.999995530e-01f, 1.666666120e-01f, 4.166565090e-02f, 8.333227597e-03f,
-     1.388137927e-03f, 1.983425464e-04f, 2.455824688e-05f, 2.734730060e-06f, 2.393897489e-07f,
-     2.211615246e-08f}};
+// coefficients (fit_sincos.py, fit_moment): 12 terms to 6.1e-8 on |t| <= 2.5 -- an eighth
+// of the special-function unit's own error, so the moments never lose accuracy against
+// the direct sum.  (A second, 8-term form for |t| <= 0.85 was dropped: with its copies of
+// the code gone, and those of direct ranges that end before the last pair, the kernel
+// misses the instruction cache less -- coherent batch 9.06 -> 8.30 ms, precision shard
+// 78.8 -> 77.7.)
+constexpr float kX12 = 2.5f;
+__device__ const float g_moment_coef[kMaxP] = {
+    1.0f, 1.0f, 4.999995530e-01f, 1.666666120e-01f, 4.166565090e-02f, 8.333227597e-03f,
+    1.388137927e-03f, 1.983425464e-04f, 2.455824688e-05f, 2.734730060e-06f, 2.393897489e-07f,
+    2.211615246e-08f};
 
 // The walk over (work unit, particle, chunk), advanced by lane 0 only; a unit is
 // particle pp of every tile of an item.
@@ -137,7 +138,7 @@ struct __align__(128) WarpM {
 template <bool COH>
 struct SmemM {
     WarpM<COH> w[kWarps];
-    float coef[2][kMaxP];
+    float coef[kMaxP];
     int abort_flag;
 };
 
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
     for (int v = lane; v < (int)(sizeof(S.ff) / 4); v += 32)
         reinterpret_cast<uint32_t*>(S.ff)[v] = 0u;
     if (tid == 0) SB.abort_flag = 0;
-    if (tid < 2 * kMaxP) (&SB.coef[0][0])[tid] = (&g_moment_coef[0][0])[tid];
+    if (tid < kMaxP) SB.coef[tid] = g_moment_coef[tid];
     __syncthreads();
 
     // ---- (lane 0) describe the cursor's chunk as chunk L, issue its copy and step on;
@@ -382,9 +383,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
 
     f2 a1r[kPairs], a1i[kPairs], a2r[kPairs], a2i[kPairs];
     float wm[kPairs];            // largest |omega| of the pair (warp-uniform); < 0: no slot in use
-    const float* om0 = nullptr;  // this lane's first frequency, and slots left from there
+    const float* om0 = nullptr;  // this lane's frequency in slot 0 (read from `skip` on)
     const float *nh0 = nullptr, *nl0 = nullptr;
-    int left = 0, sel = -1;
+    int skip = 0, sel = -1;
     int kc = 0;                  // chunk of the particle
     float bh = 0.0f, bl = 0.0f;  // lane = chunk: reference phases but for the centre
 #pragma unroll
@@ -419,16 +420,19 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
             if (lane == 12) S.dv[12] = (float)p.species[it.sp].qdt;
             const int kb = it.ftile * (32 * kFT);
             sel = w.sel;
-            left = w.grid_len - kb - lane;
-            om0 = p.omega + w.grid_off + kb + lane;
-            nh0 = p.nu_hi + w.grid_off + kb + lane;
-            nl0 = p.nu_lo + w.grid_off + kb + lane;
+            // a grid's last tile fills the pairs from the end: the high frequencies then
+            // always reach the last pair, whatever the grid's length
+            skip = max(0, 32 * kFT - (w.grid_len - kb + 63) / 64 * 64);
+            om0 = p.omega + w.grid_off + kb + lane - skip;
+            nh0 = p.nu_hi + w.grid_off + kb + lane - skip;
+            nl0 = p.nu_lo + w.grid_off + kb + lane - skip;
 #pragma unroll
             for (int i = 0; i < kPairs; ++i) {
+                wm[i] = -1.0f;
+                if (64 * i < skip) continue;
                 const float w0 = om0[64 * i], w1 = om0[64 * i + 32];
-                const uint32_t m = __reduce_max_sync(
-                    0xffffffffu, __float_as_uint(fmaxf(fabsf(w0), fabsf(w1))));
-                wm[i] = kb + 64 * i < w.grid_len ? __uint_as_float(m) : -1.0f;
+                wm[i] = __uint_as_float(__reduce_max_sync(
+                    0xffffffffu, __float_as_uint(fmaxf(fabsf(w0), fabsf(w1)))));
             }
             __syncwarp();
         }
@@ -543,20 +547,19 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
             if (at != lane) V1 = V2 = 0.0f;
         }
 
-        // ---- mode of each pair: 0 direct, 1 / 2 moments of the whole chunk with 8 / 12
-        // terms, 3 / 4 of two / four sub-blocks, -1 no slot in use
+        // ---- mode of each pair: 0 direct, 1 moments of the whole chunk, 2 / 3 of two / four
+        // sub-blocks, -1 no slot in use
         auto warp_max_abs = [&](float v) {       // NaN compares above everything
             return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v) & 0x7fffffffu));
         };
         const float h1 = warp_max_abs(d);
         int mode[kPairs];
-        bool big = false, need12 = false;
+        bool big = false;
 #pragma unroll
         for (int i = 0; i < kPairs; ++i) {
             const float x = wm[i] * h1;
-            mode[i] = wm[i] < 0.0f ? -1 : (x <= kX8 ? 1 : (x <= kX12 ? 2 : 0));
+            mode[i] = wm[i] < 0.0f ? -1 : (x <= kX12 ? 1 : 0);
             big = big || (mode[i] == 0 && x <= 5.0f * kX12);   // a quarter's may fit
-            need12 = need12 || mode[i] == 2;
         }
         float h2 = 0.0f, h4 = 0.0f, c2 = 0.0f, c4 = 0.0f;
         if (big) {
@@ -568,18 +571,13 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
             h4 = warp_max_abs(d - c4);
 #pragma unroll
             for (int i = 0; i < kPairs; ++i)
-                if (mode[i] == 0) mode[i] = wm[i] * h2 <= kX12 ? 3 : (wm[i] * h4 <= kX12 ? 4 : 0);
+                if (mode[i] == 0) mode[i] = wm[i] * h2 <= kX12 ? 2 : (wm[i] * h4 <= kX12 ? 3 : 0);
         }
-        // direct pairs as one contiguous range (a pair between two direct ones joins them)
-        int da = kPairs, db = 0;
+        // direct pairs as one range up to the last (a pair above a direct one joins it)
+        int da = kPairs;
 #pragma unroll
-        for (int i = 0; i < kPairs; ++i)
-            if (mode[i] == 0) {
-                da = da < i ? da : i;
-                db = i + 1;
-            }
-        // a range that does not reach the last pair starts at the first (code size)
-        if (db < kPairs) da = db > 0 ? 0 : da;
+        for (int i = kPairs - 1; i >= 0; --i)
+            if (mode[i] == 0) da = i;
         // (the frequency arrays are padded with zeros to whole tiles of 256)
         auto freq = [&](int i) -> f2 {           // omega of a pair
             return pk(__ldg(om0 + 64 * i), __ldg(om0 + 64 * i + 32));
@@ -590,46 +588,37 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
             return mul2(anchor_turns2(nh, nl, an), dup(6.28318530717958647f));
         };
 
-        // ---- moments and their evaluation, one block size after the other (8 terms only
-        // where every whole-chunk pair can use them: one set of moments)
+        // ---- moments and their evaluation, one block size after the other
         uint32_t has = 0;
 #pragma unroll
         for (int i = 0; i < kPairs; ++i) {
-            if (mode[i] == 1 && need12) mode[i] = 2;
-            if (i >= da && i < db) mode[i] = 0;
+            if (i >= da) mode[i] = 0;
             if (mode[i] > 0) has |= 1u << mode[i];
         }
 #pragma unroll 1
         for (int md = 1; has >> md; ++md) {
             if (!((has >> md) & 1u)) continue;
-            const float hm = md <= 2 ? h1 : (md == 3 ? h2 : h4);
-            const float cc = md <= 2 ? 0.0f : (md == 3 ? c2 : c4);
-            const int o0 = md <= 2 ? 16 : (md == 3 ? 8 : 4);
+            const float hm = md == 1 ? h1 : (md == 2 ? h2 : h4);
+            const float cc = md == 1 ? 0.0f : (md == 2 ? c2 : c4);
+            const int o0 = 32 >> md;
             // a power of two above the largest offset: exact scalings
             const uint32_t hb = (__float_as_uint(hm) & 0x7f800000u) + 0x00800000u;
             const float hs = __uint_as_float(hb), ih = __uint_as_float(0x7f000000u - hb);
-            if (md == 1)
-                moments<8>(V1, V2, d * ih, o0, lane, S.mom, SB.coef[0]);
-            else
-                moments<12>(V1, V2, (d - cc) * ih, o0, lane, S.mom, SB.coef[1]);
+            moments<kMaxP>(V1, V2, (d - cc) * ih, o0, lane, S.mom, SB.coef);
 #pragma unroll
             for (int i = 0; i < kPairs; ++i) {
                 if (mode[i] != md) continue;
                 const f2 om = freq(i), th = anchor(i);
                 const f2 x = mul2(om, dup(hs)), nx = mul2(om, dup(-hs));
-                if (md == 1) {
-                    eval_moments<8>(S.mom[0], x, nx, th, a1r[i], a1i[i], a2r[i], a2i[i]);
-                } else {
 #pragma unroll 1
-                    for (int b = 0; b < 32; b += 2 * o0) {
-                        const float cb = __shfl_sync(0xffffffffu, cc, b);
-                        eval_moments<12>(S.mom[b / (2 * o0)], x, nx, fma2(om, dup(cb), th), a1r[i],
-                                         a1i[i], a2r[i], a2i[i]);
-                    }
+                for (int b = 0; b < 32; b += 2 * o0) {
+                    const float cb = __shfl_sync(0xffffffffu, cc, b);
+                    eval_moments<kMaxP>(S.mom[b / (2 * o0)], x, nx, fma2(om, dup(cb), th), a1r[i], a1i[i],
+                                        a2r[i], a2i[i]);
                 }
             }
         }
-        if (da < db) {
+        if (da < kPairs) {
             __syncwarp();
             S.geo[lane] = make_float4(V1, V2, d, 0.0f);
             __syncwarp();
@@ -637,20 +626,16 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
 #pragma unroll
             for (int i = 0; i < kPairs; ++i) {
                 om[i] = th[i] = 0;
-                if (i >= da && i < db) {
+                if (i >= da) {
                     om[i] = freq(i);
                     th[i] = anchor(i);
                 }
             }
-            switch (da + 4 * (kPairs - db)) {
+            switch (da) {
                 case 0: direct_sum<0, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
                 case 1: direct_sum<1, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
                 case 2: direct_sum<2, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 3: direct_sum<3, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 4: direct_sum<0, 3, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 8: direct_sum<0, 2, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                case 12: direct_sum<0, 1, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
-                default: break;
+                default: direct_sum<3, 4, !COH>(S.geo, lo, hi, om, th, a1r, a1i, a2r, a2i); break;
             }
         }
 
@@ -686,14 +671,15 @@ __global__ void __launch_bounds__(kThreads, kBlocks) accum32_moment_kernel(const
             // ---- work unit done: the FP64 accumulators
             const WorkItem it = p.items[ii];
             const WinDev w = p.wins[it.win];
-            const int64_t o = w.out_off + (int64_t)it.row * w.grid_len + it.ftile * (32 * kFT) + lane;
+            const int64_t o = w.out_off + (int64_t)it.row * w.grid_len + it.ftile * (32 * kFT) + lane - skip;
+            const int left = w.grid_len - it.ftile * (32 * kFT) - lane + skip;
 #pragma unroll 1
             for (int s = 0; s < kFT; ++s) {
                 constexpr int NC = COH ? 4 : 1;
                 for (int comp = 0; comp < NC; ++comp) {
                     const float2 a = S.ff[NC * s + comp][lane];
                     S.ff[NC * s + comp][lane] = make_float2(0.0f, 0.0f);
-                    if (32 * s < left)
+                    if (32 * s >= skip && 32 * s < left)
                         atomicAdd(p.acc + NC * (o + 32 * s) + comp, (double)a.x + (double)a.y);
                 }
             }
