@@ -146,6 +146,5 @@ if __name__ == "__main__":
     print("C2, C4, C6, C8 =", ", ".join(f"{v:.9e}f" for v in C))
     print("PI_HI, PI_LO =", f"{PI_HI:.9e}f, {PI_LO:.9e}f")
     print("max |error| of e^{i theta}, |theta| <= 2000:", max_error(S, C))
-    for x0, n in ((0.85, 4), (2.5, 6)):
-        c, e = fit_moment(x0, n)
-        print(f"moments, |t| <= {x0}:", ", ".join(f"{v:.9e}f" for v in c), "max error", e)
+    c, e = fit_moment(2.5, 6)
+    print("moments, |t| <= 2.5:", ", ".join(f"{v:.9e}f" for v in c), "max error", e)

@@ -30,6 +30,12 @@
 // pairs in packed f32x2 registers (two slots per instruction).  Frequency slots
 // beyond the grid's end and particles beyond a species' count are skipped.  Particle
 // sums run in float-float per warp and reach the FP64 accumulators once per work unit.
+//
+// Against the direct kernel (which the explicit variants still run): 8195 particles x 4096
+// samples x 8 directions x 1024 omega, ingest included, 125.0 -> 77.4 ms; 1024 x 2000 x 192 x
+// 2048 356 -> 221 ms; 1024 x 2000 x 12 x 64 3.49 -> 1.35 ms.  Issue slots 58% busy, the
+// special-function pipe 63-68%, FMA 42%: dependent chains of four warps per scheduler, and the
+// instruction cache, are what is left.
 #include "rad_accum32.cuh"
 
 namespace rad {
