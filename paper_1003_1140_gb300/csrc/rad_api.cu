@@ -171,7 +171,7 @@ struct rad_ctx {
     std::vector<Event> events;     // eager: sorted by call; defer: one event
     std::map<int64_t, int> event_at;
     int64_t next_step = 0;
-    int64_t max_s1 = 0;
+    int64_t min_s0 = INT64_MAX, max_s1 = 0;   // the windows' span
     bool deferred_done = false;     // deferred windows already evaluated
 
     // timing
@@ -916,6 +916,8 @@ static IngestParams ingest_params(const rad_ctx* c)
     p.anc32 = c->anc32;
     p.ncols = c->ncols;
     p.ring = c->ring;
+    p.keep0 = c->min_s0 * c->nsub;
+    p.keep1 = c->max_s1 * c->nsub;
     p.comps = c->comps;
     p.K = c->K;
     p.nblk = c->nblk;
@@ -1472,7 +1474,6 @@ int rad_init(rad_ctx** out, const double* dirs, int32_t D, const double* freqs,
     c->n_in = c->in_off.back();
     c->ncols = std::max<int64_t>(col, kTileP);
     if (c->ncols > (int64_t)1 << 30) return bail(RAD_EINVAL);
-    int64_t min_s0 = INT64_MAX;
     for (int w = 0; w < n_win; ++w) {
         const rad_window& W = win[w];
         if (W.s0 < 0 || W.s1 < W.s0 || W.freq_grid < 0 || W.freq_grid >= n_grids ||
@@ -1496,11 +1497,11 @@ int rad_init(rad_ctx** out, const double* dirs, int32_t D, const double* freqs,
         c->out_len += (int64_t)wd.size() * grid_len[W.freq_grid];
         c->win_dirs.push_back(std::move(wd));
         c->max_s1 = std::max<int64_t>(c->max_s1, W.s1);
-        min_s0 = std::min<int64_t>(min_s0, W.s0);
+        c->min_s0 = std::min<int64_t>(c->min_s0, W.s0);
     }
     // ring length: longest window (eager) or the whole span (defer is decided
     // later, so size for the span; the ring is what the windows need at once)
-    int64_t span = std::max<int64_t>(1, c->max_s1 - min_s0);
+    int64_t span = std::max<int64_t>(1, c->max_s1 - c->min_s0);
     c->ring = (span + 31) / 32 * 32 + 64;
 
     int rc;

@@ -112,6 +112,12 @@ __device__ uint32_t selector_bits(const IngestParams& p, const double x[3], cons
     return bits;
 }
 
+// Whether a chunk is inside the windows' span (see IngestParams).
+__device__ __forceinline__ bool kept(const IngestParams& p, int64_t chunk)
+{
+    return (chunk + 1) * kChunk32 > p.keep0 && chunk * kChunk32 < p.keep1;
+}
+
 // Component 0 of a sample in either ring (components are kChunk32 apart).
 template <class T>
 __device__ __forceinline__ T* slab_at(T* slab, const IngestParams& p, int64_t tile, int64_t slot,
@@ -267,6 +273,7 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                     rk[c] = rp[c] + p.dt * (tau / 6.0) * (b0[c] + 4.0 * bh[c] + bk[c]);
                 }
                 const int64_t M = m * p.nsub + k;
+                if (!kept(p, M / kChunk32)) continue;
                 const int64_t sl = M % p.ring;
                 if (p.slab32) {
                     float* an = p.anc32 + ((tile * p.nblk + (M / p.K) % p.nblk) * kTileP + pp) * 6;
@@ -307,6 +314,8 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                     if (p.comps > kCompsPlain) o[10 * kChunk32] = (double)flags;
                 }
             }
+        } else if (!kept(p, m / kChunk32)) {
+            // no window needs the sample
         } else if (p.slab32) {
             // FP32 ring: the only cancellation-prone quantities are differenced
             // in FP64 -- du = u_{m+1/2} - u_{m-1/2} and r_m - r_anchor -- and the
@@ -597,6 +606,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
         const int64_t m = q * kChunk32 + sm, slot0 = (int64_t)rc * kChunk32;
         if (++rc == (uint32_t)(p.ring / kChunk32)) rc = 0;
         const bool valid = m >= b.m0 && m <= b.m1;
+        const bool keep = kept(p, q);
 #pragma unroll
         for (int c = 0; c < 3; ++c) row(m, sm, c);
         if (tid < 3 * kTileP) row(q * kChunk32 + kChunk32, kChunk32, tid >> 3);
@@ -624,7 +634,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                 for (int c = 0; c < 3; ++c) n[c] -= jc[r][c][pp];
         }
         // anchors: r_a as an FP32 hi + lo pair; offsets are relative to exactly hi + lo
-        if (MODE != 2 && sm % p.K == 0) {
+        if (MODE != 2 && keep && sm % p.K == 0) {
             float* an = p.anc32 + ((tile * p.nblk + (slot0 + sm) / p.K) * kTileP + pp) * 6;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -650,7 +660,9 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
             moved[tid >> 3][pp] = t;                     // zero beyond the last call
         }
         if (any) __syncthreads();
-        if (MODE == 2) {
+        if (!keep) {
+            // no window needs the chunk
+        } else if (MODE == 2) {
             // beta at the half steps, once per call (a sample uses two neighbouring ones):
             // one reciprocal square root where the samples took three square roots and
             // ten divisions between them (154 FP64 instructions each)

@@ -230,6 +230,10 @@ struct IngestParams {
     float* anc32;           // FP32 path: tile-major anchor ring (r_a as hi + lo)
     int64_t ncols;
     int64_t ring;           // samples in the ring
+    // chunks that hold samples [keep0, keep1) go into the ring, others only carry the
+    // particle state on: the ring is as long as the windows' span, so two chunks outside
+    // it may share a slot, and blocks of one launch would write it in no order
+    int64_t keep0, keep1;
     int32_t comps;          // ring components per sample (10, or 11 with selector flags)
     int32_t K;              // anchor interval (FP32 path)
     int64_t nblk;           // anchor blocks in the ring

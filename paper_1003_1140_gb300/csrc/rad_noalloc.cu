@@ -219,6 +219,8 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     ip.anc32 = reinterpret_cast<float*>(B + o_anc);
     ip.ncols = ncols;
     ip.ring = ring;
+    ip.keep0 = 0;
+    ip.keep1 = S;
     ip.comps = kCompsPlain;
     ip.K = K;
     ip.nblk = nblk;
