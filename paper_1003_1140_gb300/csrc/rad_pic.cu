@@ -7,9 +7,11 @@
 //      moves x to n+1 and deposits the charge-conserving current of the move
 //      (Esirkepov's decomposition for linear shapes on the 3 x 3 nodes the old
 //      and new positions share) with FP64 atomics, then wraps x;
-//   2. ampere:  E^{n+1} = E^n + dt (curl B^{n+1/2} - J^{n+1/2}) with
-//      B^{n+1/2} = B^n - dt/2 curl E^n formed on the fly, J cleared;
-//   3. faraday: B^{n+1} = B^n - dt/2 curl E^n - dt/2 curl E^{n+1}.
+//   2. ampere:  E^{n+1} = E^n + dt (curl B^{n+1/2} - J^{n+1/2}), J cleared;
+//   3. faraday: B^{n+1} = B^{n+1/2} - dt/2 curl E^{n+1}, and with the same curl
+//      B^{n+3/2} = B^{n+1} - dt/2 curl E^{n+1}, kept beside B^{n+1}.
+// All fields are updated in place, at fixed addresses: a captured step can be replayed,
+// also with direct steps between the replays.
 // FP64 throughout (the diagnostic's FP64 parity chain reaches back into the
 // particle state); a PIC step costs about 200 FP64 operations per particle,
 // which this GPU's FP64 pipe (1/64 of FP32) sustains at about two billion
@@ -20,7 +22,6 @@
 #include <cmath>
 #include <cstdio>
 #include <new>
-#include <utility>
 #include <string>
 #include <vector>
 
@@ -223,36 +224,29 @@ __device__ __forceinline__ double curl_fwd(const double* __restrict__ F, int64_t
     return -(F[qjp] - F[q]) * inv_d;
 }
 
-// E1 = E + dt (curl B' - J) with B' = B - c curl E (c = dt / 2) formed at the points
-// it is needed; J is left at zero for the next step's deposit.
-__global__ void ampere(const double* __restrict__ E, const double* __restrict__ B,
-                       double* __restrict__ J, double* __restrict__ E1, int n, double inv_d, double dt)
+// E += dt (curl Bh - J) with Bh the magnetic field at the half step; J is left at zero for
+// the next step's deposit.
+__global__ void ampere(double* __restrict__ E, const double* __restrict__ Bh, double* __restrict__ J,
+                       int n, double inv_d, double dt)
 {
     const int64_t nn = (int64_t)n * n;
-    const double c = 0.5 * dt;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nn;
          q += (int64_t)gridDim.x * blockDim.x) {
         const int j = (int)(q / n), k = (int)(q - (int64_t)j * n);
-        const int64_t jp = j + 1 == n ? n - nn : n, jm = j == 0 ? nn - n : -n;   // row steps
-        const int kp = k + 1 == n ? 1 - n : 1, km = k == 0 ? n - 1 : -1;
-        auto half = [&](int comp, int64_t r, int64_t rjp, int64_t rkp) {
-            return B[comp * nn + r] - c * curl_fwd(E, nn, comp, r, rjp, rkp, inv_d);
-        };
-        const int64_t qjm = q + jm, qkm = q + km;
-        const double bx = half(0, q, q + jp, q + kp), bxj = half(0, qjm, q, qjm + kp),
-                     bxk = half(0, qkm, qkm + jp, q);
-        const double by = half(1, q, q + jp, q + kp), byk = half(1, qkm, qkm + jp, q);
-        const double bz = half(2, q, q + jp, q + kp), bzj = half(2, qjm, q, qjm + kp);
-        E1[q] = E[q] + dt * ((bz - bzj) * inv_d - (by - byk) * inv_d - J[q]);
-        E1[nn + q] = E[nn + q] + dt * ((bx - bxk) * inv_d - J[nn + q]);
-        E1[2 * nn + q] = E[2 * nn + q] + dt * (-(bx - bxj) * inv_d - J[2 * nn + q]);
+        const int64_t qjm = j == 0 ? q + nn - n : q - n, qkm = k == 0 ? q + n - 1 : q - 1;
+        const double bx = Bh[q], by = Bh[nn + q], bz = Bh[2 * nn + q];
+        const double bxj = Bh[qjm], bxk = Bh[qkm], byk = Bh[nn + qkm], bzj = Bh[2 * nn + qjm];
+        E[q] = E[q] + dt * ((bz - bzj) * inv_d - (by - byk) * inv_d - J[q]);
+        E[nn + q] = E[nn + q] + dt * ((bx - bxk) * inv_d - J[nn + q]);
+        E[2 * nn + q] = E[2 * nn + q] + dt * (-(bx - bxj) * inv_d - J[2 * nn + q]);
         J[q] = J[nn + q] = J[2 * nn + q] = 0.0;
     }
 }
 
-// B -= c curl E0 (first half step), then B -= c curl E1 (second), c = dt / 2.
-__global__ void faraday(const double* __restrict__ E0, const double* __restrict__ E1,
-                        double* __restrict__ B, int n, double inv_d, double c)
+// With c = dt / 2 and the new E: B = Bh - c curl E (the second half of this step), then
+// Bh = B - c curl E (the first half of the next one, which starts from the same E).
+__global__ void faraday(const double* __restrict__ E, double* __restrict__ B, double* __restrict__ Bh,
+                        int n, double inv_d, double c)
 {
     const int64_t nn = (int64_t)n * n;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nn;
@@ -261,11 +255,26 @@ __global__ void faraday(const double* __restrict__ E0, const double* __restrict_
         const int64_t qjp = j + 1 == n ? q + n - nn : q + n, qkp = k + 1 == n ? q + 1 - n : q + 1;
 #pragma unroll
         for (int comp = 0; comp < 3; ++comp) {
-            double b = B[comp * nn + q];
-            b -= c * curl_fwd(E0, nn, comp, q, qjp, qkp, inv_d);
-            b -= c * curl_fwd(E1, nn, comp, q, qjp, qkp, inv_d);
+            const double r = curl_fwd(E, nn, comp, q, qjp, qkp, inv_d);
+            const double b = Bh[comp * nn + q] - c * r;
             B[comp * nn + q] = b;
+            Bh[comp * nn + q] = b - c * r;
         }
+    }
+}
+
+// Bh = B - c curl E of fields that were set from outside.
+__global__ void half_step(const double* __restrict__ E, const double* __restrict__ B,
+                          double* __restrict__ Bh, int n, double inv_d, double c)
+{
+    const int64_t nn = (int64_t)n * n;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nn;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        const int j = (int)(q / n), k = (int)(q - (int64_t)j * n);
+        const int64_t qjp = j + 1 == n ? q + n - nn : q + n, qkp = k + 1 == n ? q + 1 - n : q + 1;
+#pragma unroll
+        for (int comp = 0; comp < 3; ++comp)
+            Bh[comp * nn + q] = B[comp * nn + q] - c * curl_fwd(E, nn, comp, q, qjp, qkp, inv_d);
     }
 }
 
@@ -338,8 +347,8 @@ bool is_dev(const void* ptr)
 struct rad_pic {
     PicDev dev{};
     double* E = nullptr;
-    double* E1 = nullptr;       // E of the next step (the two swap)
     double* B = nullptr;
+    double* Bh = nullptr;       // B half a step on (B - dt/2 curl E)
     double* J = nullptr;
     double* x = nullptr;
     double* u = nullptr;
@@ -383,11 +392,9 @@ static int pic_fields(rad_pic* p, cudaStream_t st)
     const int64_t nn = (int64_t)p->dev.n * p->dev.n;
     const double inv_d = p->dev.inv_d, dt = p->dev.dt;
     const unsigned cells = (unsigned)((nn + 127) / 128);
-    ampere<<<cells, 128, 0, st>>>(p->E, p->B, p->J, p->E1, p->dev.n, inv_d, dt);
-    faraday<<<cells, 128, 0, st>>>(p->E, p->E1, p->B, p->dev.n, inv_d, 0.5 * dt);
+    ampere<<<cells, 128, 0, st>>>(p->E, p->Bh, p->J, p->dev.n, inv_d, dt);
+    faraday<<<cells, 128, 0, st>>>(p->E, p->B, p->Bh, p->dev.n, inv_d, 0.5 * dt);
     PCU(cudaGetLastError());
-    std::swap(p->E, p->E1);
-    p->dev.E = p->E;
     ++p->steps;
     return RAD_PIC_OK;
 }
@@ -427,8 +434,8 @@ int rad_pic_init(rad_pic** out, int32_t n, double d, double dt, const rad_pic_sp
         }                                                                             \
     } while (0)
     PMAL(p->E, 3 * nn * sizeof(double));
-    PMAL(p->E1, 3 * nn * sizeof(double));
     PMAL(p->B, 3 * nn * sizeof(double));
+    PMAL(p->Bh, 3 * nn * sizeof(double));
     PMAL(p->J, 3 * nn * sizeof(double));
     PMAL(p->x, 3 * N * sizeof(double));
     PMAL(p->u, 3 * N * sizeof(double));
@@ -437,6 +444,7 @@ int rad_pic_init(rad_pic** out, int32_t n, double d, double dt, const rad_pic_sp
 #undef PMAL
     if (cudaMemset(p->E, 0, 3 * nn * sizeof(double)) != cudaSuccess ||
         cudaMemset(p->B, 0, 3 * nn * sizeof(double)) != cudaSuccess ||
+        cudaMemset(p->Bh, 0, 3 * nn * sizeof(double)) != cudaSuccess ||
         cudaMemset(p->J, 0, 3 * nn * sizeof(double)) != cudaSuccess ||
         (N > 0 && (cudaMemcpy(p->x, x, 3 * N * sizeof(double), cudaMemcpyDefault) != cudaSuccess ||
                    cudaMemcpy(p->u, u, 3 * N * sizeof(double), cudaMemcpyDefault) != cudaSuccess)))
@@ -480,6 +488,9 @@ int rad_pic_set_fields(rad_pic* p, const double* E, const double* B)
     const size_t bytes = 3 * (size_t)p->dev.n * p->dev.n * sizeof(double);
     if (E) PCU(cudaMemcpyAsync(p->E, E, bytes, cudaMemcpyDefault, p->st));
     if (B) PCU(cudaMemcpyAsync(p->B, B, bytes, cudaMemcpyDefault, p->st));
+    half_step<<<grid_for((int64_t)p->dev.n * p->dev.n), 256, 0, p->st>>>(
+        p->E, p->B, p->Bh, p->dev.n, p->dev.inv_d, 0.5 * p->dev.dt);
+    PCU(cudaGetLastError());
     PCU(cudaStreamSynchronize(p->st));
     return RAD_PIC_OK;
 }
@@ -638,7 +649,7 @@ void rad_pic_destroy(rad_pic* p)
 {
     if (!p) return;
     if (p->st) cudaStreamSynchronize(p->st);
-    for (double* q : {p->E, p->E1, p->B, p->J, p->x, p->u, p->mw, p->en, p->xt, p->ut})
+    for (double* q : {p->E, p->B, p->Bh, p->J, p->x, p->u, p->mw, p->en, p->xt, p->ut})
         if (q) cudaFree(q);
     if (p->staged_ev) cudaEventDestroy(p->staged_ev);
     if (p->read_ev) cudaEventDestroy(p->read_ev);
