@@ -19,6 +19,7 @@
 // segment's starting image count is the launch's initial count plus the integer
 // changes of the earlier segments (wind kernels), so the split changes no result.
 #include <algorithm>
+#include <climits>
 
 #include "rad_internal.cuh"
 
@@ -32,7 +33,27 @@ namespace rad {
 __device__ __forceinline__ double image_jump(double d, double L, double half_L)
 {
     if (!(L > 0.0) || fabs(d) <= half_L) return 0.0;
-    return rint(d / L);
+    const double j = rint(d / L);
+    return fabs(j) < 1073741824.0 ? j : __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// Image counts as integers; kLost stands for NaN and stays.
+constexpr int kLost = INT_MIN;
+__device__ __forceinline__ int as_count(double v)
+{
+    return fabs(v) < 2147483648.0 ? (int)v : kLost;
+}
+__device__ __forceinline__ int add_count(int a, int b)
+{
+    return a == kLost || b == kLost ? kLost : a + b;
+}
+__device__ __forceinline__ int sub_count(int a, int b)
+{
+    return a == kLost || b == kLost ? kLost : a - b;
+}
+__device__ __forceinline__ double from_count(int n)
+{
+    return n == kLost ? __longlong_as_double(0x7ff8000000000000ll) : (double)n;
 }
 
 // Calls [s_begin, s_end) of segment g of the launch.
@@ -79,7 +100,7 @@ __global__ void __launch_bounds__(256) wind_kernel(const IngestParams p)
     for (int64_t s = s_begin; s < s_end; ++s) {
         for (int c = 0; c < 3; ++c) {
             const double xn = p.x[(s - p.step0) * 3 * ld + c * ld + xi];
-            if (have) dn[c] -= (int32_t)image_jump(xn - xp[c], p.box_L, half_L);
+            if (have) dn[c] = sub_count(dn[c], as_count(image_jump(xn - xp[c], p.box_L, half_L)));
             xp[c] = xn;
         }
         have = true;
@@ -175,7 +196,7 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
         for (int c = 0; c < 3; ++c) {
             // image count at the launch start, plus the earlier segments' changes
             double n0 = p.step0 > 0 ? p.r_prev[c * nc + col] : 0.0;
-            for (int h = 0; h < g; ++h) n0 += (double)p.wind[((int64_t)h * 3 + c) * cnt + k];
+            for (int h = 0; h < g; ++h) n0 += from_count(p.wind[((int64_t)h * 3 + c) * cnt + k]);
             off[c] = box ? p.box_L * n0 : 0.0;
             if (g == 0) {
                 xp[c] = p.x_prev[c * nc + col];
@@ -491,7 +512,7 @@ __device__ __forceinline__ int64_t tile_particle(const IngestParams& p, int64_t 
 // took 60 us for 1024 particles x 2000 calls, a chain of 28 load rounds).
 __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
 {
-    __shared__ int tot[3][kTileP];
+    __shared__ int tot[3][kTileP], lost[3][kTileP];
     const int tid = threadIdx.x, pp = tid & (kTileP - 1);
     const int tile_l = (int)(blockIdx.x % p.n_tiles), g = (int)(blockIdx.x / p.n_tiles);
     const int64_t col = (p.tile0 + tile_l) * kTileP + pp;
@@ -501,7 +522,7 @@ __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
     const BatchRange b = batch_range(p);
     const float lim = 0.4999f * (float)p.box_L;
     const double half_L = 0.5 * p.box_L;
-    if (tid < 3 * kTileP) tot[tid >> 3][pp] = 0;
+    if (tid < 3 * kTileP) tot[tid >> 3][pp] = lost[tid >> 3][pp] = 0;
     __syncthreads();
     int dn[3] = {0, 0, 0};
     if (i >= 0) {
@@ -527,18 +548,23 @@ __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         if (maybe_jump(xp[k], xn[u][k], lim))
-                            dn[k] -= (int)image_jump(xn[u][k] - xp[k], p.box_L, half_L);
+                            dn[k] = sub_count(dn[k], as_count(image_jump(xn[u][k] - xp[k], p.box_L, half_L)));
                         xp[k] = xn[u][k];
                     }
             }
         }
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-            if (dn[k]) atomicAdd(&tot[k][pp], dn[k]);
+        for (int k = 0; k < 3; ++k) {
+            if (dn[k] == kLost)
+                lost[k][pp] = 1;
+            else if (dn[k])
+                atomicAdd(&tot[k][pp], dn[k]);
+        }
     }
     __syncthreads();
     if (tid < 3 * kTileP && i >= 0)
-        p.wind[((int64_t)g * 3 + (tid >> 3)) * npart + (i - p.first)] = tot[tid >> 3][pp];
+        p.wind[((int64_t)g * 3 + (tid >> 3)) * npart + (i - p.first)] =
+            lost[tid >> 3][pp] ? kLost : tot[tid >> 3][pp];
 }
 
 // One block: chunks [q0, q1) (32 samples each) of one 8-particle tile, thread = sample
@@ -581,8 +607,9 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
         const int c = tid >> 3;
         int n = 0;
         if (box && i >= 0) {
-            if (p.step0 > 0) n = (int)p.r_prev[c * p.ncols + col];
-            for (int h = 0; h < g; ++h) n += p.wind[((int64_t)h * 3 + c) * npart + (i - p.first)];
+            if (p.step0 > 0) n = as_count(p.r_prev[c * p.ncols + col]);
+            for (int h = 0; h < g; ++h)
+                n = add_count(n, p.wind[((int64_t)h * 3 + c) * npart + (i - p.first)]);
         }
         cnt[c][pp] = n;
     }
@@ -627,12 +654,19 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
 #pragma unroll
             for (int c = 0; c < 3; ++c)
                 jc[sm][c][pp] =
-                    jump ? (int)image_jump(xs[sm + 1][c][pp] - x[c], p.box_L, 0.5 * p.box_L) : 0;
+                    jump ? as_count(image_jump(xs[sm + 1][c][pp] - x[c], p.box_L, 0.5 * p.box_L)) : 0;
             __syncthreads();
+            int t[3] = {0, 0, 0}, low[3] = {n[0], n[1], n[2]};   // kLost is the lowest value
             for (int r = 0; r < sm; ++r)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) n[c] -= jc[r][c][pp];
+                for (int c = 0; c < 3; ++c) {
+                    t[c] += jc[r][c][pp];
+                    low[c] = min(low[c], jc[r][c][pp]);
+                }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) n[c] = low[c] == kLost ? kLost : n[c] - t[c];
         }
+        auto off = [&](int c) { return p.box_L * from_count(n[c]); };
         // anchors: r_a as an FP32 hi + lo pair; offsets are relative to exactly hi + lo
         if (MODE != 2 && keep && sm % p.K == 0) {
             float* an = p.anc32 + ((tile * p.nblk + (slot0 + sm) / p.K) * kTileP + pp) * 6;
@@ -640,7 +674,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
             for (int c = 0; c < 3; ++c) {
                 float hi = 0.0f, lo = 0.0f;
                 if (valid && i >= 0) {
-                    const double r = x[c] + p.box_L * (double)n[c];
+                    const double r = x[c] + off(c);
                     hi = (float)r;
                     lo = (float)(r - (double)hi);
                     an[c] = hi;
@@ -650,14 +684,17 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                     lo = an[3 + c];
                 }
                 const double ra = (double)hi + (double)lo;
-                ras[sm / p.K][c][pp] = any ? ra : ra - p.box_L * (double)n[c];
+                ras[sm / p.K][c][pp] = any ? ra : ra - off(c);
             }
         }
         __syncthreads();                                 // ras; jc read by everyone
         if (any && tid < 3 * kTileP) {
-            int t = 0;
-            for (int r = 0; r < kChunk32; ++r) t += jc[r][tid >> 3][pp];
-            moved[tid >> 3][pp] = t;                     // zero beyond the last call
+            int t = 0, low = 0;
+            for (int r = 0; r < kChunk32; ++r) {
+                t += jc[r][tid >> 3][pp];
+                low = min(low, jc[r][tid >> 3][pp]);
+            }
+            moved[tid >> 3][pp] = low == kLost ? kLost : t;   // zero beyond the last call
         }
         if (any) __syncthreads();
         if (!keep) {
@@ -679,7 +716,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                 const double igb = inv_gamma(ub[0], ub[1], ub[2]);
                 double* o = slab_at(p.slab64, p, tile, slot0 + sm, pp);
                 for (int c = 0; c < 3; ++c) {
-                    o[c * kChunk32] = n[c] ? __dadd_rn(x[c], __dmul_rn(p.box_L, (double)n[c])) : x[c];
+                    o[c * kChunk32] = n[c] ? __dadd_rn(x[c], off(c)) : x[c];
                     o[(3 + c) * kChunk32] = ub[c] * igb;
                     o[(6 + c) * kChunk32] = __dmul_rn(__dsub_rn(bh[sm + 1][c][pp], bh[sm][c][pp]), idt64);
                 }
@@ -698,7 +735,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const double ra = ras[sm / p.K][c][pp];
-                const double d = any ? (x[c] + p.box_L * (double)n[c]) - ra : x[c] - ra;
+                const double d = any ? (x[c] + off(c)) - ra : x[c] - ra;
                 const float dh = (float)d;
                 o[c * kChunk32] = dh;
                 if (MODE == 1) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
@@ -745,7 +782,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
             // the launch's last call is the state carried on (staged when other blocks
             // of the launch may still be reading the state arrays)
             const int c = tid >> 3, r = (int)(b.s1 - q * kChunk32);
-            const double nn = (double)(cnt[c][pp] - (any ? moved[c][pp] : 0));
+            const double nn = from_count(sub_count(cnt[c][pp], any ? moved[c][pp] : 0));
             const int64_t k = i - p.first;
             double* sx = p.n_seg > 1 ? p.state_out + c * npart + k : p.x_prev + c * p.ncols + col;
             double* sr = p.n_seg > 1 ? p.state_out + (3 + c) * npart + k : p.r_prev + c * p.ncols + col;
@@ -755,7 +792,8 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
             *su = us[r][c][pp];
         }
         __syncthreads();
-        if (any && tid < 3 * kTileP) cnt[tid >> 3][pp] -= moved[tid >> 3][pp];
+        if (any && tid < 3 * kTileP)
+            cnt[tid >> 3][pp] = sub_count(cnt[tid >> 3][pp], moved[tid >> 3][pp]);
     }
     if (bad) atomicOr(p.err_word, kErrNaN);
 }
