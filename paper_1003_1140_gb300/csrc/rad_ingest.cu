@@ -478,6 +478,12 @@ __device__ __forceinline__ bool maybe_jump(double a, double b, float lim)
     return !(fmaf(fmaxf(fabsf(fa), fabsf(fb)), 1.9073486e-6f, fabsf(fb - fa)) <= lim);
 }
 
+// maybe_jump's limit; boxes whose lengths leave the float range take the exact test always.
+__device__ __forceinline__ float crossing_limit(double L)
+{
+    return L > 1e-30 && L < 1e30 ? 0.4999f * (float)L : -1.0f;
+}
+
 // Geometry of a batched launch: samples [m0, m1], chunks [c0, c1], calls up to s1.
 struct BatchRange {
     int64_t m0, m1, s1, c0, c1;
@@ -520,7 +526,7 @@ __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
     const int64_t npart = p.count ? p.count : p.n_in - p.first;
     const int64_t ld = p.ld ? p.ld : p.n_in;
     const BatchRange b = batch_range(p);
-    const float lim = 0.4999f * (float)p.box_L;
+    const float lim = crossing_limit(p.box_L);
     const double half_L = 0.5 * p.box_L;
     if (tid < 3 * kTileP) tot[tid >> 3][pp] = lost[tid >> 3][pp] = 0;
     __syncthreads();
@@ -597,7 +603,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
     const int64_t q0 = b.c0 + (int64_t)g * p.seg_len;
     const int64_t q1 = min(q0 + p.seg_len, b.c1 + 1);
     const bool box = p.box_L > 0.0;
-    const float lim = 0.4999f * (float)p.box_L;
+    const float lim = crossing_limit(p.box_L);
     const double idt64 = 1.0 / p.dt;
     const float idt = (float)idt64;
     const int ostride = p.comps * kChunk32 + 4;
