@@ -171,6 +171,7 @@ struct rad_ctx {
     std::vector<Event> events;     // eager: sorted by call; defer: one event
     std::map<int64_t, int> event_at;
     int64_t next_step = 0;
+    int64_t sm0 = 0, sm1 = -1;      // chunks of the FP32 ring that are slot-major: [sm0, sm1]
     int64_t min_s0 = INT64_MAX, max_s1 = 0;   // the windows' span
     bool deferred_done = false;     // deferred windows already evaluated
 
@@ -836,11 +837,14 @@ static int32_t take_stall(rad_ctx* c)
     return s ? 1 : 0;
 }
 
+static int to_particle_major(rad_ctx* c);
 static int launch_event(rad_ctx* c, Event& ev)
 {
     if (ev.items.empty()) return RAD_OK;
     int32_t few = 0;
     const int grid = event_grid(c, ev, &few);
+    const int rc = to_particle_major(c);
+    if (rc) return rc;
     cudaEvent_t e0 = next_event(c->acc_ev, c->acc_used, true);
     CU(cudaEventRecord(e0, c->stream));
     cudaError_t e;
@@ -907,7 +911,9 @@ static IngestParams ingest_params(const rad_ctx* c)
     IngestParams p{};
     p.n_in = c->n_in;
     p.dt = c->dt;
+    p.idt = 1.0 / c->dt;
     p.box_L = c->box_L;
+    p.lim = crossing_limit(c->box_L);
     p.x_prev = c->x_prev;
     p.r_prev = c->r_prev;
     p.u_prev = c->u_prev;
@@ -916,8 +922,8 @@ static IngestParams ingest_params(const rad_ctx* c)
     p.anc32 = c->anc32;
     p.ncols = c->ncols;
     p.ring = c->ring;
-    p.keep0 = c->min_s0 * c->nsub;
-    p.keep1 = c->max_s1 * c->nsub;
+    p.keep0 = c->min_s0 * c->nsub / kChunk32 * kChunk32;
+    p.keep1 = (c->max_s1 * c->nsub + kChunk32 - 1) / kChunk32 * kChunk32;
     p.comps = c->comps;
     p.K = c->K;
     p.nblk = c->nblk;
@@ -930,6 +936,40 @@ static IngestParams ingest_params(const rad_ctx* c)
     p.n_sel = c->n_sel;
     p.nsub = c->nsub;
     return p;
+}
+
+// The slot-major chunks of the FP32 ring to particle-major.
+static int to_particle_major(rad_ctx* c)
+{
+    if (c->sm1 < c->sm0) return RAD_OK;
+    CU(particle_major(c->slab32, c->ncols, c->ring, c->comps, c->sm0, c->sm1, c->stream));
+    c->sm1 = c->sm0 - 1;
+    return RAD_OK;
+}
+
+// The layout of the chunks that a launch over all particles writes, and the record of it.
+static int chunk_layout(rad_ctx* c, IngestParams& p)
+{
+    p.slot_major0 = p.slot_major = 0;
+    if (c->precision != RAD_FP32_SPLIT) return RAD_OK;
+    const int64_t m0 = std::max<int64_t>(0, p.step0 - 1) * c->nsub;
+    const int64_t m1 = (p.step0 + p.n_steps - 1) * c->nsub - 1;    // (before m0: no sample yet)
+    const int64_t c0 = m0 / kChunk32;
+    p.slot_major = !ingest_batched(p);
+    // a chunk that earlier calls began keeps its layout
+    p.slot_major0 = m0 % kChunk32 ? c->sm0 <= c->sm1 && c->sm1 == c0 : p.slot_major;
+    const int64_t lo = std::max(p.slot_major0 ? c0 : c0 + 1, p.keep0 / kChunk32);
+    const int64_t hi = m1 < m0 ? -1
+                               : std::min(p.slot_major ? m1 / kChunk32 : c0, p.keep1 / kChunk32 - 1);
+    if (lo > hi) return RAD_OK;
+    if (c->sm0 <= c->sm1 && lo <= c->sm1 + 1) {
+        c->sm1 = std::max(c->sm1, hi);
+        return RAD_OK;
+    }
+    const int rc = to_particle_major(c);
+    c->sm0 = lo;
+    c->sm1 = hi;
+    return rc;
 }
 
 // Scratch of a time-segmented ingest launch over count particles and n_steps
@@ -980,6 +1020,7 @@ static int ingest_device(rad_ctx* c, int64_t step0, int64_t n, const double* x, 
         p.step0 = s;
         p.n_steps = (int32_t)(stop - s);
         int rs = seg_scratch(c, c->n_in, stop - s, p);
+        if (!rs) rs = chunk_layout(c, p);
         if (rs) return rs;
         cudaEvent_t e0 = nullptr;
         if (c->time_ingest) {
@@ -1110,6 +1151,7 @@ static int ingest_host_blocked(rad_ctx* c, int64_t step0, int64_t n, const doubl
         ppb = std::max(ppb, tot);
     }
     int rc = blocked_lists(c, bounds);
+    if (!rc) rc = to_particle_major(c);   // (the blocks' launches write turned chunks)
     if (rc) return rc;
     const size_t cap = c->opt.reserved[2] > 0 ? (size_t)c->opt.reserved[2] << 20 : kBlockStageBytes;
     const int64_t chunk = std::max<int64_t>(1, (int64_t)(cap / (6 * ppb * sizeof(double))));
@@ -1126,6 +1168,7 @@ static int ingest_host_blocked(rad_ctx* c, int64_t step0, int64_t n, const doubl
         c->bstage_bytes = need;
     }
     IngestParams p = ingest_params(c);
+    p.turned = 1;
     const int64_t end = step0 + n;
     int64_t s = step0;
     while (s < end) {
@@ -1285,6 +1328,9 @@ static int step_via_graph(rad_ctx* c, int64_t step, const double* x, const doubl
     }
     StepGraph* g = nullptr;
     int rc = graph_for(c, kind, p, &g);
+    if (rc) return rc;
+    // (a closing step's graph accumulates: its one sample goes in particle-major)
+    rc = kind > 0 ? to_particle_major(c) : chunk_layout(c, p);
     if (rc) return rc;
     cudaKernelNodeParams kp;
     CU(cudaGraphKernelNodeGetParams(g->ingest_node, &kp));
@@ -1821,6 +1867,7 @@ int rad_next_shard(rad_ctx* c)
     // the ring, anchors and per-particle ingest state are rewritten from step 0
     // by the next shard's calls; the accumulators keep their sums
     c->next_step = 0;
+    c->sm1 = c->sm0 - 1;
     c->deferred_done = false;
     return RAD_OK;
 }
@@ -1833,6 +1880,7 @@ int rad_reset(rad_ctx* c)
     CU(cudaMemsetAsync(c->acc, 0, std::max<size_t>(1, acc_n) * sizeof(double), c->stream));
     CU(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
     c->next_step = 0;
+    c->sm1 = c->sm0 - 1;
     c->deferred_done = false;
     return RAD_OK;
 }

@@ -14,7 +14,12 @@
 //     8-particle tile into ring records, one thread per sample, and writes each
 //     record as one contiguous block;
 //   * ingest_kernel (a few calls, or sub-cycling): a thread walks one particle
-//     through one time segment of the launch's steps.
+//     through one time segment of the launch's steps.  One call's sample of a particle
+//     would be ten 4-byte stores to as many sectors of the sample-innermost ring (181 us
+//     per call of 557,056 particles); the chunk that is being filled is slot-major
+//     instead, eight particles to a sector, and turned when a window closes (76 us, and
+//     6.6 us per call for turning it; 135 us with four FP64 divisions per call and
+//     particle and the slot-major ring of before).
 // Both split a launch in time when the particles alone leave the GPU idle: a later
 // segment's starting image count is the launch's initial count plus the integer
 // changes of the earlier segments (wind kernels), so the split changes no result.
@@ -35,6 +40,32 @@ __device__ __forceinline__ double image_jump(double d, double L, double half_L)
     if (!(L > 0.0) || fabs(d) <= half_L) return 0.0;
     const double j = rint(d / L);
     return fabs(j) < 1073741824.0 ? j : __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// The binary exponent and leading 20 mantissa bits of a double as a float (truncated;
+// magnitudes below the float range become 0, above it infinity): integer work only.
+__device__ __forceinline__ float coarse(double v)
+{
+    const int hi = __double2hiint(v);
+    const int t = (hi & 0x7fffffff) - (896 << 20);
+    const uint32_t m = t <= 0 ? 0u : (t >= (255 << 20) ? 0x7f800000u : (uint32_t)t << 3);
+    return __uint_as_float(m | ((uint32_t)hi & 0x80000000u));
+}
+
+// False only if the displacement b - a is surely within half a box (no crossing): the
+// difference of the coarse values plus their truncation (2^-20 of each) against
+// 0.4999 L.  Keeps the 1/64-rate FP64 pipe out of the common case.
+__device__ __forceinline__ bool maybe_jump(double a, double b, float lim)
+{
+    const float fa = coarse(a), fb = coarse(b);
+    return !(fmaf(fmaxf(fabsf(fa), fabsf(fb)), 1.9073486e-6f, fabsf(fb - fa)) <= lim);
+}
+
+// maybe_jump's limit for a box (on the host: FP64 work, also once per block, shows in the
+// kernels' time); boxes whose lengths leave the float range take the exact test always.
+float crossing_limit(double L)
+{
+    return L > 1e-30 && L < 1e30 ? 0.4999f * (float)L : -1.0f;
 }
 
 // Image counts as integers; kLost stands for NaN and stays.
@@ -133,12 +164,6 @@ __device__ uint32_t selector_bits(const IngestParams& p, const double x[3], cons
     return bits;
 }
 
-// Whether a chunk is inside the windows' span (see IngestParams).
-__device__ __forceinline__ bool kept(const IngestParams& p, int64_t chunk)
-{
-    return (chunk + 1) * kChunk32 > p.keep0 && chunk * kChunk32 < p.keep1;
-}
-
 // Component 0 of a sample in either ring (components are kChunk32 apart).
 template <class T>
 __device__ __forceinline__ T* slab_at(T* slab, const IngestParams& p, int64_t tile, int64_t slot,
@@ -155,13 +180,15 @@ __device__ __forceinline__ double inv_gamma(double a, double b, double c)
     return rsqrt(fma(a, a, fma(b, b, fma(c, c, 1.0))));
 }
 
-// 64-thread blocks (launch_ingest), at least 8 resident per SM: the FP64-bound
-// loop needs the warps to hide its latency more than it needs registers.
-// PRING: the ring is the precise-phase one (comps >= kCompsPrec), which also
-// takes the lo part of each position offset -- a build of its own, so that the
-// FP64-bound common build carries none of that work.
-template <bool PRING>
-__global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
+// 64-thread blocks (launch_ingest), 7 of them resident per SM: 146 registers hold the loop
+// without spilling, and the warps left hide its FP64 latency (557,056 particles, us per call
+// of 512-call batches / of single calls: 6 blocks 24.0 / 85.7, 7 26.2 / 78.7, 8 30.6 / 81.7;
+// the FP64 instructions alone would take 17).
+// MODE as in ingest_tile_kernel (1, the precise-phase ring, also takes the lo part of each
+// position offset), SUB sub-cycled samples: builds of their own, so that the common one
+// carries none of that work and none of its registers.
+template <int MODE, bool SUB>
+__global__ void __launch_bounds__(64, SUB ? 6 : 7) ingest_kernel(const IngestParams p)
 {
     const int64_t cnt = p.count ? p.count : p.n_in - p.first;
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -182,22 +209,39 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
     const int64_t nc = p.ncols;
     const int64_t tile = col / kTileP, pp = col % kTileP;
 
-    double xp[3], off[3], rp[3], up[3], ra[3];   // off = L n (n the image count), exact
+    double xp[3], off[3], rp[3], up[3], ra[3];   // off = L n
+    int img[3];                          // image counts n
     const double half_L = 0.5 * p.box_L;
     const bool box = p.box_L > 0.0;
-    bool have_state = s_begin > 0;
-    // ring slot, position in the anchor block and anchor block of the next
-    // sample m (nsub = 1), advanced by counters instead of 64-bit divisions
-    int64_t m_next = s_begin > 0 ? s_begin - 1 : 0;
-    // (nblk is 0 for an FP64 ring, which has no anchors)
-    int64_t slot_n = m_next % p.ring, kpos_n = m_next % p.K;
-    int64_t blk_n = p.nblk > 0 ? (m_next / p.K) % p.nblk : 0;
+    const float lim = p.lim;
+    const float idt = (float)p.idt;
+    const bool have_state = s_begin > 0;
+    // ring slot, position in the anchor block and anchor block of the next sample
+    // (nsub = 1), advanced by counters instead of 64-bit divisions (a ring has far
+    // fewer than 2^31 samples; nblk is 0 for an FP64 ring, which has no anchors)
+    const int64_t m_next = s_begin > 0 ? s_begin - 1 : 0;
+    const int ring = (int)p.ring, nblk = (int)p.nblk;
+    int slot_n = (int)(m_next % p.ring), kpos_n = (int)(m_next % p.K);
+    int blk_n = p.nblk > 0 ? (int)((m_next / p.K) % p.nblk) : 0;
+    // this thread's calls whose sample the ring takes: [keep_a, keep_b)
+    const int keep_a = (int)min(max(p.keep0 + 1 - s_begin, int64_t(0)), int64_t(n_loc));
+    const int keep_b = (int)min(max(p.keep1 + 1 - s_begin, int64_t(0)), int64_t(n_loc));
+    // the current chunk's layout (a chunk that starts here takes the launch's)
+    bool sm = g == 0 ? p.slot_major0 : p.slot_major;
+    // component 0 of a sample in FP32 ring slot `slot`; os: from component to component
+    auto slab32_at = [&](int64_t slot, int& os) {
+        if (slot % kChunk32 == 0) sm = p.slot_major;
+        os = sm ? kTileP : kChunk32;
+        return sm ? p.slab32 + (tile * p.ring + slot) * (p.comps * kTileP) + pp
+                  : slab_at(p.slab32, p, tile, slot, pp);
+    };
     if (have_state) {
         for (int c = 0; c < 3; ++c) {
             // image count at the launch start, plus the earlier segments' changes
-            double n0 = p.step0 > 0 ? p.r_prev[c * nc + col] : 0.0;
-            for (int h = 0; h < g; ++h) n0 += from_count(p.wind[((int64_t)h * 3 + c) * cnt + k]);
-            off[c] = box ? p.box_L * n0 : 0.0;
+            img[c] = box && p.step0 > 0 ? as_count(p.r_prev[c * nc + col]) : 0;
+            for (int h = 0; h < g && box; ++h)
+                img[c] = add_count(img[c], p.wind[((int64_t)h * 3 + c) * cnt + k]);
+            off[c] = box ? p.box_L * from_count(img[c]) : 0.0;
             if (g == 0) {
                 xp[c] = p.x_prev[c * nc + col];
                 up[c] = p.u_prev[c * nc + col];
@@ -208,36 +252,38 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             rp[c] = xp[c] + off[c];
         }
     }
-    bool have_anchor = false;
+    bool have_anchor = false, have_uf = false;
+    float uf[3] = {0.0f, 0.0f, 0.0f};    // FP32 ring: u of the last sample's later call
     bool bad = false;
 
     // the next step's inputs are loaded while this step is being processed
     double xq[3], uq[3];
+    const double *xs = p.x + t0 * 3 * ld + xi, *us = p.u + t0 * 3 * ld + xi;
     for (int c = 0; c < 3; ++c) {
-        xq[c] = n_loc > 0 ? p.x[t0 * 3 * ld + c * ld + xi] : 0.0;
-        uq[c] = n_loc > 0 ? p.u[t0 * 3 * ld + c * ld + xi] : 0.0;
+        xq[c] = n_loc > 0 ? xs[c * ld] : 0.0;
+        uq[c] = n_loc > 0 ? us[c * ld] : 0.0;
     }
     for (int t = 0; t < n_loc; ++t) {
-        const int64_t s = s_begin + t;
         double xn[3], un[3], rn[3];
         for (int c = 0; c < 3; ++c) {
             xn[c] = xq[c];
             un[c] = uq[c];
         }
         if (t + 1 < n_loc) {
-            const double* xs = p.x + (t0 + t + 1) * 3 * ld;
-            const double* us = p.u + (t0 + t + 1) * 3 * ld;
+            xs += 3 * ld;
+            us += 3 * ld;
             for (int c = 0; c < 3; ++c) {
-                xq[c] = xs[c * ld + xi];
-                uq[c] = us[c * ld + xi];
+                xq[c] = xs[c * ld];
+                uq[c] = us[c * ld];
             }
         }
         if (p.check) {
             for (int c = 0; c < 3; ++c) bad |= !isfinite(xn[c]) || !isfinite(un[c]);
         }
-        if (s == 0) {
+        if (!have_state && t == 0) {     // call 0
             for (int c = 0; c < 3; ++c) {
                 xp[c] = xn[c];
+                img[c] = 0;
                 off[c] = 0.0;
                 rp[c] = xn[c];
                 up[c] = un[c];
@@ -245,22 +291,25 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             continue;
         }
         // unwrapped position of this call: r = x + L n, n counting box crossings
-        // (L n, exact, changes only at a crossing)
         for (int c = 0; c < 3; ++c) {
-            const double jump = image_jump(xn[c] - xp[c], p.box_L, half_L);
-            if (jump != 0.0) off[c] -= p.box_L * jump;      // exact: integer multiples of L
+            if (box && maybe_jump(xp[c], xn[c], lim)) {
+                const double jump = image_jump(xn[c] - xp[c], p.box_L, half_L);
+                if (jump != 0.0) {
+                    img[c] = sub_count(img[c], as_count(jump));
+                    off[c] = p.box_L * from_count(img[c]);
+                }
+            }
             rn[c] = xn[c] + off[c];
         }
 
         // sample m = s - 1: r_m = rp, u_{m-1/2} = up, u_{m+1/2} = un
-        const int64_t m = s - 1;
-        const int64_t slot = slot_n, kpos = kpos_n, blk = blk_n;
-        if (++slot_n == p.ring) slot_n = 0;
+        const int slot = slot_n, kpos = kpos_n, blk = blk_n;
+        if (++slot_n == ring) slot_n = 0;
         if (++kpos_n == p.K) {
             kpos_n = 0;
-            if (++blk_n == p.nblk) blk_n = 0;
+            if (++blk_n == nblk) blk_n = 0;
         }
-        if (p.nsub > 1) {
+        if (SUB) {
             // Sub-cycling (Sec. 2.2: tracked particles sub-cycled at
             // dt_synth <= dt_sim / 10): n sub-samples per PIC sample at
             // tau = (k + 1/2)/n - 1/2, u(tau) = ubar + tau du linear in time
@@ -276,6 +325,7 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             const double g0 = sqrt(1.0 + (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]));
             for (int c = 0; c < 3; ++c) b0[c] = ub[c] / g0;
             const uint32_t flags = p.n_sel ? selector_bits(p, xp, ub) : 0xffffffffu;
+            const int64_t m = s_begin + t - 1;
             for (int k = 0; k < p.nsub; ++k) {
                 const double tau = (k + 0.5) / p.nsub - 0.5;
                 double uk[3], uh[3], bk[3], bh[3], bd[3], rk[3];
@@ -294,9 +344,9 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                     rk[c] = rp[c] + p.dt * (tau / 6.0) * (b0[c] + 4.0 * bh[c] + bk[c]);
                 }
                 const int64_t M = m * p.nsub + k;
-                if (!kept(p, M / kChunk32)) continue;
+                if (M < p.keep0 || M >= p.keep1) continue;
                 const int64_t sl = M % p.ring;
-                if (p.slab32) {
+                if (MODE != 2) {
                     float* an = p.anc32 + ((tile * p.nblk + (M / p.K) % p.nblk) * kTileP + pp) * 6;
                     if ((M % p.K) == 0 || !have_anchor) {
                         if ((M % p.K) == 0) {
@@ -313,17 +363,18 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                         }
                         have_anchor = true;
                     }
-                    float* o = slab_at(p.slab32, p, tile, sl, pp);
+                    int os;
+                    float* o = slab32_at(sl, os);
                     for (int c = 0; c < 3; ++c) {
                         const double d = rk[c] - ra[c];
                         const float dh = (float)d;
-                        o[c * kChunk32] = dh;
-                        if (PRING) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
-                        o[(3 + c) * kChunk32] = (float)bk[c];
-                        o[(6 + c) * kChunk32] = (float)bd[c];
+                        o[c * os] = dh;
+                        if (MODE == 1) o[(11 + c) * os] = (float)(d - (double)dh);
+                        o[(3 + c) * os] = (float)bk[c];
+                        o[(6 + c) * os] = (float)bd[c];
                     }
-                    o[9 * kChunk32] = (float)(1.0 / gk2);
-                    if (p.comps > kCompsPlain) o[10 * kChunk32] = __uint_as_float(flags);
+                    o[9 * os] = (float)(1.0 / gk2);
+                    if (p.comps > kCompsPlain) o[10 * os] = __uint_as_float(flags);
                 } else {
                     double* o = slab_at(p.slab64, p, tile, sl, pp);
                     for (int c = 0; c < 3; ++c) {
@@ -335,9 +386,9 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                     if (p.comps > kCompsPlain) o[10 * kChunk32] = (double)flags;
                 }
             }
-        } else if (!kept(p, m / kChunk32)) {
+        } else if (t < keep_a || t >= keep_b) {
             // no window needs the sample
-        } else if (p.slab32) {
+        } else if (MODE != 2) {
             // FP32 ring: the only cancellation-prone quantities are differenced
             // in FP64 -- du = u_{m+1/2} - u_{m-1/2} and r_m - r_anchor -- and the
             // rest is evaluated in FP32 through the rearrangement
@@ -362,11 +413,12 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             }
             float um[3], uq[3], du[3], ub[3];
             for (int c = 0; c < 3; ++c) {
-                um[c] = (float)up[c];
-                uq[c] = (float)un[c];
+                um[c] = have_uf ? uf[c] : (float)up[c];
+                uq[c] = uf[c] = (float)un[c];
                 du[c] = (float)(un[c] - up[c]);
                 ub[c] = 0.5f * (um[c] + uq[c]);
             }
+            have_uf = true;
             const float gm = sqrtf(1.0f + (um[0] * um[0] + um[1] * um[1] + um[2] * um[2]));
             const float gq = sqrtf(1.0f + (uq[0] * uq[0] + uq[1] * uq[1] + uq[2] * uq[2]));
             const float gb2 = 1.0f + (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
@@ -375,39 +427,39 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
                               du[2] * (uq[2] + um[2]);
             const float igq = 1.0f / gq;
             const float corr = dus / (gq * gm * (gq + gm));
-            const float idt = (float)(1.0 / p.dt);
-            float* o = slab_at(p.slab32, p, tile, slot, pp);
+            int os;
+            float* o = slab32_at(slot, os);
             for (int c = 0; c < 3; ++c) {
                 const double d = rp[c] - ra[c];
                 const float dh = (float)d;
-                o[c * kChunk32] = dh;
+                o[c * os] = dh;
                 // precise-phase ring: the rounding of the offset as its lo part
-                if (PRING) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
+                if (MODE == 1) o[(11 + c) * os] = (float)(d - (double)dh);
             }
-            o[3 * kChunk32] = ub[0] * igb;
-            o[4 * kChunk32] = ub[1] * igb;
-            o[5 * kChunk32] = ub[2] * igb;
-            o[6 * kChunk32] = (du[0] * igq - um[0] * corr) * idt;
-            o[7 * kChunk32] = (du[1] * igq - um[1] * corr) * idt;
-            o[8 * kChunk32] = (du[2] * igq - um[2] * corr) * idt;
-            o[9 * kChunk32] = 1.0f / gb2;
+            o[3 * os] = ub[0] * igb;
+            o[4 * os] = ub[1] * igb;
+            o[5 * os] = ub[2] * igb;
+            o[6 * os] = (du[0] * igq - um[0] * corr) * idt;
+            o[7 * os] = (du[1] * igq - um[1] * corr) * idt;
+            o[8 * os] = (du[2] * igq - um[2] * corr) * idt;
+            o[9 * os] = 1.0f / gb2;
             if (p.comps > kCompsPlain) {
                 double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
                                  __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
                                  __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
-                o[10 * kChunk32] = __uint_as_float(p.n_sel ? selector_bits(p, xp, ubd) : 0xffffffffu);
+                o[10 * os] = __uint_as_float(p.n_sel ? selector_bits(p, xp, ubd) : 0xffffffffu);
             }
         } else {
             double ub[3];
             for (int c = 0; c < 3; ++c) ub[c] = 0.5 * (up[c] + un[c]);
             const double igm = inv_gamma(up[0], up[1], up[2]), igp = inv_gamma(un[0], un[1], un[2]);
-            const double igb = inv_gamma(ub[0], ub[1], ub[2]), idt64 = 1.0 / p.dt;
+            const double igb = inv_gamma(ub[0], ub[1], ub[2]);
             double* o = slab_at(p.slab64, p, tile, slot, pp);
             for (int c = 0; c < 3; ++c) {
                 o[c * kChunk32] = rp[c];
                 o[(3 + c) * kChunk32] = ub[c] * igb;
                 o[(6 + c) * kChunk32] =
-                    __dmul_rn(__dsub_rn(__dmul_rn(un[c], igp), __dmul_rn(up[c], igm)), idt64);
+                    __dmul_rn(__dsub_rn(__dmul_rn(un[c], igp), __dmul_rn(up[c], igm)), p.idt);
             }
             o[9 * kChunk32] = igb * igb;
             if (p.comps > kCompsPlain) {
@@ -428,13 +480,13 @@ __global__ void __launch_bounds__(64, 8) ingest_kernel(const IngestParams p)
             // segment 0 may still be reading the state arrays: stage it
             for (int c = 0; c < 3; ++c) {
                 p.state_out[c * cnt + k] = xp[c];
-                p.state_out[(3 + c) * cnt + k] = box ? off[c] / p.box_L : 0.0;   // exact
+                p.state_out[(3 + c) * cnt + k] = box ? from_count(img[c]) : 0.0;
                 p.state_out[(6 + c) * cnt + k] = up[c];
             }
         } else {
             for (int c = 0; c < 3; ++c) {
                 p.x_prev[c * nc + col] = xp[c];
-                p.r_prev[c * nc + col] = box ? off[c] / p.box_L : 0.0;
+                p.r_prev[c * nc + col] = box ? from_count(img[c]) : 0.0;
                 p.u_prev[c * nc + col] = up[c];
             }
         }
@@ -457,31 +509,6 @@ __global__ void store_state(const IngestParams p)
         p.r_prev[c * p.ncols + col] = p.state_out[(3 + c) * cnt + k];
         p.u_prev[c * p.ncols + col] = p.state_out[(6 + c) * cnt + k];
     }
-}
-
-// The binary exponent and leading 20 mantissa bits of a double as a float (truncated;
-// magnitudes below the float range become 0, above it infinity): integer work only.
-__device__ __forceinline__ float coarse(double v)
-{
-    const int hi = __double2hiint(v);
-    const int t = (hi & 0x7fffffff) - (896 << 20);
-    const uint32_t m = t <= 0 ? 0u : (t >= (255 << 20) ? 0x7f800000u : (uint32_t)t << 3);
-    return __uint_as_float(m | ((uint32_t)hi & 0x80000000u));
-}
-
-// False only if the displacement b - a is surely within half a box (no crossing): the
-// difference of the coarse values plus their truncation (2^-20 of each) against
-// 0.4999 L.  Keeps the 1/64-rate FP64 pipe out of the common case.
-__device__ __forceinline__ bool maybe_jump(double a, double b, float lim)
-{
-    const float fa = coarse(a), fb = coarse(b);
-    return !(fmaf(fmaxf(fabsf(fa), fabsf(fb)), 1.9073486e-6f, fabsf(fb - fa)) <= lim);
-}
-
-// maybe_jump's limit; boxes whose lengths leave the float range take the exact test always.
-__device__ __forceinline__ float crossing_limit(double L)
-{
-    return L > 1e-30 && L < 1e30 ? 0.4999f * (float)L : -1.0f;
 }
 
 // Geometry of a batched launch: samples [m0, m1], chunks [c0, c1], calls up to s1.
@@ -526,7 +553,7 @@ __global__ void __launch_bounds__(256) tile_wind_kernel(const IngestParams p)
     const int64_t npart = p.count ? p.count : p.n_in - p.first;
     const int64_t ld = p.ld ? p.ld : p.n_in;
     const BatchRange b = batch_range(p);
-    const float lim = crossing_limit(p.box_L);
+    const float lim = p.lim;
     const double half_L = 0.5 * p.box_L;
     if (tid < 3 * kTileP) tot[tid >> 3][pp] = lost[tid >> 3][pp] = 0;
     __syncthreads();
@@ -603,9 +630,8 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
     const int64_t q0 = b.c0 + (int64_t)g * p.seg_len;
     const int64_t q1 = min(q0 + p.seg_len, b.c1 + 1);
     const bool box = p.box_L > 0.0;
-    const float lim = crossing_limit(p.box_L);
-    const double idt64 = 1.0 / p.dt;
-    const float idt = (float)idt64;
+    const float lim = p.lim;
+    const float idt = (float)p.idt;
     const int ostride = p.comps * kChunk32 + 4;
     bool bad = false;
 
@@ -639,7 +665,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
         const int64_t m = q * kChunk32 + sm, slot0 = (int64_t)rc * kChunk32;
         if (++rc == (uint32_t)(p.ring / kChunk32)) rc = 0;
         const bool valid = m >= b.m0 && m <= b.m1;
-        const bool keep = kept(p, q);
+        const bool keep = q * kChunk32 >= p.keep0 && q * kChunk32 < p.keep1;
 #pragma unroll
         for (int c = 0; c < 3; ++c) row(m, sm, c);
         if (tid < 3 * kTileP) row(q * kChunk32 + kChunk32, kChunk32, tid >> 3);
@@ -656,23 +682,34 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
         // image counts: the chunk's starting count unless something crossed in it
         const bool any = __syncthreads_or(jump);
         int n[3] = {cnt[0][pp], cnt[1][pp], cnt[2][pp]};
+        bool gone = false;               // a crossing count of the chunk is kLost
         if (any) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-                jc[sm][c][pp] =
+            for (int c = 0; c < 3; ++c) {
+                const int j =
                     jump ? as_count(image_jump(xs[sm + 1][c][pp] - x[c], p.box_L, 0.5 * p.box_L)) : 0;
-            __syncthreads();
-            int t[3] = {0, 0, 0}, low[3] = {n[0], n[1], n[2]};   // kLost is the lowest value
-            for (int r = 0; r < sm; ++r)
+                jc[sm][c][pp] = j;
+                gone |= j == kLost;
+            }
+            gone = __syncthreads_or(gone);
+            if (!gone) {
+                for (int r = 0; r < sm; ++r)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    t[c] += jc[r][c][pp];
-                    low[c] = min(low[c], jc[r][c][pp]);
-                }
+                    for (int c = 0; c < 3; ++c) n[c] -= jc[r][c][pp];
+            } else {
+#pragma unroll 1
+                for (int r = 0; r < sm; ++r)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) n[c] = low[c] == kLost ? kLost : n[c] - t[c];
+                    for (int c = 0; c < 3; ++c) n[c] = sub_count(n[c], jc[r][c][pp]);
+            }
         }
-        auto off = [&](int c) { return p.box_L * from_count(n[c]); };
+        // a lost count makes the position NaN (its own count then is of no interest)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (cnt[c][pp] == kLost || n[c] == kLost) {
+                x[c] = __longlong_as_double(0x7ff8000000000000ll);
+                n[c] = 0;
+            }
         // anchors: r_a as an FP32 hi + lo pair; offsets are relative to exactly hi + lo
         if (MODE != 2 && keep && sm % p.K == 0) {
             float* an = p.anc32 + ((tile * p.nblk + (slot0 + sm) / p.K) * kTileP + pp) * 6;
@@ -680,7 +717,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
             for (int c = 0; c < 3; ++c) {
                 float hi = 0.0f, lo = 0.0f;
                 if (valid && i >= 0) {
-                    const double r = x[c] + off(c);
+                    const double r = x[c] + p.box_L * (double)n[c];
                     hi = (float)r;
                     lo = (float)(r - (double)hi);
                     an[c] = hi;
@@ -690,17 +727,19 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                     lo = an[3 + c];
                 }
                 const double ra = (double)hi + (double)lo;
-                ras[sm / p.K][c][pp] = any ? ra : ra - off(c);
+                ras[sm / p.K][c][pp] = any ? ra : ra - p.box_L * (double)n[c];
             }
         }
         __syncthreads();                                 // ras; jc read by everyone
         if (any && tid < 3 * kTileP) {
-            int t = 0, low = 0;
-            for (int r = 0; r < kChunk32; ++r) {
-                t += jc[r][tid >> 3][pp];
-                low = min(low, jc[r][tid >> 3][pp]);
+            int t = 0;
+            if (!gone) {
+                for (int r = 0; r < kChunk32; ++r) t += jc[r][tid >> 3][pp];
+            } else {
+#pragma unroll 1
+                for (int r = 0; r < kChunk32; ++r) t = add_count(t, jc[r][tid >> 3][pp]);
             }
-            moved[tid >> 3][pp] = low == kLost ? kLost : t;   // zero beyond the last call
+            moved[tid >> 3][pp] = t;                     // zero beyond the last call
         }
         if (any) __syncthreads();
         if (!keep) {
@@ -722,16 +761,17 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                 const double igb = inv_gamma(ub[0], ub[1], ub[2]);
                 double* o = slab_at(p.slab64, p, tile, slot0 + sm, pp);
                 for (int c = 0; c < 3; ++c) {
-                    o[c * kChunk32] = n[c] ? __dadd_rn(x[c], off(c)) : x[c];
+                    o[c * kChunk32] = n[c] ? __dadd_rn(x[c], __dmul_rn(p.box_L, (double)n[c])) : x[c];
                     o[(3 + c) * kChunk32] = ub[c] * igb;
-                    o[(6 + c) * kChunk32] = __dmul_rn(__dsub_rn(bh[sm + 1][c][pp], bh[sm][c][pp]), idt64);
+                    o[(6 + c) * kChunk32] = __dmul_rn(__dsub_rn(bh[sm + 1][c][pp], bh[sm][c][pp]), p.idt);
                 }
                 o[9 * kChunk32] = igb * igb;
                 if (p.comps > kCompsPlain) {
                     double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
                                      __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
                                      __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
-                    o[10 * kChunk32] = (double)(p.n_sel ? selector_bits(p, x, ubd) : 0xffffffffu);
+                    const double xraw[3] = {xs[sm][0][pp], xs[sm][1][pp], xs[sm][2][pp]};
+                    o[10 * kChunk32] = (double)(p.n_sel ? selector_bits(p, xraw, ubd) : 0xffffffffu);
                 }
             }
         } else {
@@ -741,7 +781,7 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const double ra = ras[sm / p.K][c][pp];
-                const double d = any ? (x[c] + off(c)) - ra : x[c] - ra;
+                const double d = any ? (x[c] + p.box_L * (double)n[c]) - ra : x[c] - ra;
                 const float dh = (float)d;
                 o[c * kChunk32] = dh;
                 if (MODE == 1) o[(11 + c) * kChunk32] = (float)(d - (double)dh);
@@ -768,7 +808,8 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                 double ubd[3] = {__dmul_rn(0.5, __dadd_rn(up[0], un[0])),
                                  __dmul_rn(0.5, __dadd_rn(up[1], un[1])),
                                  __dmul_rn(0.5, __dadd_rn(up[2], un[2]))};
-                o[10 * kChunk32] = __uint_as_float(p.n_sel ? selector_bits(p, x, ubd) : 0xffffffffu);
+                const double xraw[3] = {xs[sm][0][pp], xs[sm][1][pp], xs[sm][2][pp]};
+                o[10 * kChunk32] = __uint_as_float(p.n_sel ? selector_bits(p, xraw, ubd) : 0xffffffffu);
             }
             __syncthreads();
             float* dst = p.slab32 + (tile * p.ring + slot0) * (p.comps * kTileP);
@@ -779,7 +820,10 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
                     reinterpret_cast<float4*>(dst)[v] =
                         *reinterpret_cast<const float4*>(outs + r * ostride + 4 * w);
                 }
-            } else if (valid) {                          // the chunk's samples of this launch only
+            } else if (valid && q == b.c0 && p.slot_major0) {   // this launch's samples only,
+                for (int c = 0; c < p.comps; ++c)               // in the chunk's layout
+                    dst[(sm * p.comps + c) * kTileP + pp] = outs[pp * ostride + c * kChunk32 + sm];
+            } else if (valid) {
                 for (int c = 0; c < p.comps; ++c)
                     dst[pp * rec + c * kChunk32 + sm] = outs[pp * ostride + c * kChunk32 + sm];
             }
@@ -806,8 +850,81 @@ __global__ void __launch_bounds__(256, MODE == 0 ? 4 : 2) ingest_tile_kernel(con
 
 IngestKernels ingest_kernel_ptr()
 {
-    return {reinterpret_cast<const void*>(&ingest_kernel<false>),
-            reinterpret_cast<const void*>(&ingest_kernel<true>)};
+    return {{reinterpret_cast<const void*>(&ingest_kernel<0, false>),
+             reinterpret_cast<const void*>(&ingest_kernel<1, false>),
+             reinterpret_cast<const void*>(&ingest_kernel<0, true>),
+             reinterpret_cast<const void*>(&ingest_kernel<1, true>)}};
+}
+
+// Tiles of a launch's particles: all columns, or the range's (whole tiles of one species).
+static void tile_range(IngestParams& q)
+{
+    q.tile0 = 0;
+    q.n_tiles = (int32_t)(q.ncols / kTileP);
+    if (q.count || q.first) {
+        const int64_t cnt = q.count ? q.count : q.n_in - q.first;
+        int sp = 0;
+        while (sp + 1 < q.n_species && q.first >= q.in_off[sp + 1]) ++sp;
+        const int64_t col = q.col_off[sp] + (q.first - q.in_off[sp]);
+        q.tile0 = col / kTileP;
+        q.n_tiles = (int32_t)((col + cnt - 1) / kTileP - q.tile0 + 1);
+    }
+}
+
+// Batches of calls go through ingest_tile_kernel, a few calls (and sub-cycled samples)
+// through ingest_kernel.  A batch costs the tile kernel a round per chunk and 608 tiles (4
+// blocks on each SM), also for a chunk it fills in part only, so the shortest batch that pays
+// grows with the tiles.  FP32, us per call, tile kernel / ingest_kernel: 8000 particles,
+// batches of 16 calls 2.15 / 2.02, 32 1.38 / 1.78; 20,000, 64 2.17 / 1.86, 128 1.80 / 1.78
+// (and 0.24 for turning the chunks); from about 40,000 particles on (512 calls 2.79 / 2.38 and
+// 0.47; 65,536 4.38 / 3.31 and 0.77) never.  FP64, where ingest_kernel's three reciprocal
+// square roots per sample cost most: 65,536, 16 calls 17.8 / 13.2, 32 12.4 / 12.9, 512
+// 7.4 / 12.2.  Launches that may not leave slot-major chunks behind take the tile kernel
+// from 8 calls on.
+bool ingest_batched(const IngestParams& p)
+{
+    if (p.nsub > 1 || p.n_steps < 8) return false;
+    if (p.turned) return true;
+    IngestParams q = p;
+    tile_range(q);
+    const int64_t least = 20 * (int64_t)q.n_tiles / kSegMaxTiles - 12;
+    if (!q.slab32) return p.n_steps >= std::min<int64_t>(32, least);
+    return p.n_steps >= least && q.n_tiles < 4000;
+}
+
+// Slot-major chunks of the FP32 ring to particle-major, in place: a block per tile and chunk.
+__global__ void __launch_bounds__(256) particle_major_kernel(float* slab, int n_tiles, int64_t rchunks,
+                                                             int comps, int64_t c0)
+{
+    __shared__ float buf[kTileP * kCompsPrec * (kChunk32 + 1)];   // [particle][comp][slot], padded
+    const int64_t tile = blockIdx.x % n_tiles, c = c0 + blockIdx.x / n_tiles;
+    const int rec = comps * kChunk32, n4 = rec * kTileP / 4;
+    float4* chunk = reinterpret_cast<float4*>(slab + (tile * rchunks + c % rchunks) * (rec * kTileP));
+    for (int v = threadIdx.x; v < n4; v += 256) {
+        const float4 a = chunk[v];
+        const int q = v >> 1, slot = q / comps, comp = q - slot * comps, p = (v & 1) * 4;
+        float* o = buf + (p * comps + comp) * (kChunk32 + 1) + slot;
+        const int step = comps * (kChunk32 + 1);
+        o[0] = a.x;
+        o[step] = a.y;
+        o[2 * step] = a.z;
+        o[3 * step] = a.w;
+    }
+    __syncthreads();
+    for (int v = threadIdx.x; v < n4; v += 256) {
+        const float* i = buf + (v >> 3) * (kChunk32 + 1) + (v & 7) * 4;
+        chunk[v] = make_float4(i[0], i[1], i[2], i[3]);
+    }
+}
+
+cudaError_t particle_major(float* slab, int64_t ncols, int64_t ring, int comps, int64_t c0, int64_t c1,
+                           cudaStream_t st)
+{
+    const int64_t n_tiles = ncols / kTileP, per = std::max<int64_t>(1, (int64_t(1) << 30) / n_tiles);
+    for (; c0 <= c1; c0 += per)
+        particle_major_kernel<<<(unsigned)(n_tiles * std::min(per, c1 - c0 + 1)), 256, 0, st>>>(
+            slab, (int)n_tiles, ring / kChunk32, comps, c0);
+    return cudaGetLastError();
 }
 
 // A batch of calls through ingest_tile_kernel.
@@ -815,17 +932,7 @@ static cudaError_t launch_batch(IngestParams q, int64_t cnt, cudaStream_t st)
 {
     const BatchRange b = batch_range(q);
     const int64_t chunks = b.c1 - b.c0 + 1;
-    // tiles of the launch's particles: all columns, or the range's (whole tiles of one
-    // species)
-    q.tile0 = 0;
-    q.n_tiles = (int32_t)(q.ncols / kTileP);
-    if (q.count || q.first) {
-        int sp = 0;
-        while (sp + 1 < q.n_species && q.first >= q.in_off[sp + 1]) ++sp;
-        const int64_t col = q.col_off[sp] + (q.first - q.in_off[sp]);
-        q.tile0 = col / kTileP;
-        q.n_tiles = (int32_t)((col + cnt - 1) / kTileP - q.tile0 + 1);
-    }
+    tile_range(q);
     // Time segments (whole chunks) until the launch has about 8 blocks for every SM; from
     // 608 tiles (4 blocks per SM) on the tiles alone do, and the extra pass over x for
     // the image counts costs more than the shorter blocks give.
@@ -857,9 +964,7 @@ cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st)
     if (cnt <= 0 || p.n_steps == 0) return cudaSuccess;
     IngestParams q = p;
     q.n_seg = 1;
-    // batches of calls; a few calls (below a quarter of a chunk) keep one thread per
-    // particle, and the sub-cycled samples their own loop
-    if (p.nsub <= 1 && p.n_steps >= 8) return launch_batch(q, cnt, st);
+    if (ingest_batched(p)) return launch_batch(q, cnt, st);
     // time segments only when the particles alone leave the GPU idle: with
     // 32,768 or more one thread per particle already keeps the FP64 pipes of
     // all SMs busy, and the segments' extra pass only adds work (measured)
@@ -890,10 +995,11 @@ cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st)
         wind_kernel<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(q);
     }
     const int64_t blocks = (cnt * q.n_seg + threads - 1) / threads;
-    if (q.slab32 && q.comps >= kCompsPrec)
-        ingest_kernel<true><<<(unsigned)blocks, threads, 0, st>>>(q);
-    else
-        ingest_kernel<false><<<(unsigned)blocks, threads, 0, st>>>(q);
+    const int mode = !q.slab32 ? 2 : (q.comps >= kCompsPrec ? 1 : 0);
+    const auto kernel =
+        q.nsub > 1 ? (mode == 2 ? ingest_kernel<2, true> : mode == 1 ? ingest_kernel<1, true> : ingest_kernel<0, true>)
+                   : (mode == 2 ? ingest_kernel<2, false> : mode == 1 ? ingest_kernel<1, false> : ingest_kernel<0, false>);
+    kernel<<<(unsigned)blocks, threads, 0, st>>>(q);
     if (q.n_seg > 1) store_state<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(q);
     return cudaGetLastError();
 }

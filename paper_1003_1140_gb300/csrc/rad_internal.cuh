@@ -19,6 +19,9 @@ namespace rad {
 // chunk = (tile * ring + slot) / 32, so that a warp reads one particle's chunk
 // (contiguous, 1280 B in FP32) with lane = sample; the chunk of all eight particles is
 // one contiguous block too.
+// A chunk of the FP32 ring that single calls are filling is slot-major instead,
+// [slot % 32][c][p], until a window closes: one call's values of a tile then are whole
+// 32-byte sectors.  particle_major() turns it, in place, before the accumulation.
 // comps is 10, or 11 when sample selectors are defined (the flags word); the
 // precise-phase FP32 path adds dr's lo part as components 11-13 (comps 14).
 // FP32 split path: slab[tile][chunk][p][c][slot % 32] float, c = 0..9 (10) =
@@ -220,8 +223,9 @@ struct IngestParams {
     int64_t n_in;           // particles on the input axis
     int32_t n_steps;
     int64_t step0;          // absolute step of the first state in x/u
-    double dt;
+    double dt, idt;         // idt = 1 / dt
     double box_L;           // 0: no unwrapping
+    float lim;              // crossing_limit(box_L)
     double* x_prev;         // [3][ncols] raw x of the previous call
     double* r_prev;         // [3][ncols] image count n of the previous call (r = x + L n)
     double* u_prev;         // [3][ncols] u of the previous call
@@ -230,10 +234,14 @@ struct IngestParams {
     float* anc32;           // FP32 path: tile-major anchor ring (r_a as hi + lo)
     int64_t ncols;
     int64_t ring;           // samples in the ring
-    // chunks that hold samples [keep0, keep1) go into the ring, others only carry the
+    // samples [keep0, keep1) -- whole chunks -- go into the ring, others only carry the
     // particle state on: the ring is as long as the windows' span, so two chunks outside
     // it may share a slot, and blocks of one launch would write it in no order
     int64_t keep0, keep1;
+    // FP32 ring: whether the chunk of the launch's first sample, and those after it, are
+    // slot-major (the first one's layout may be an earlier launch's choice)
+    int32_t slot_major0, slot_major;
+    int32_t turned;         // all chunks are to be particle-major
     int32_t comps;          // ring components per sample (10, or 11 with selector flags)
     int32_t K;              // anchor interval (FP32 path)
     int64_t nblk;           // anchor blocks in the ring
@@ -317,13 +325,21 @@ struct Accum64Params {
 constexpr int kSegMaxTiles = 608;
 constexpr int64_t kSegMaxParticles = 32768;
 cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st);
-// The two builds of the ingest kernel (common ring, precise-phase ring); a
-// kernel function pointer compares equal to the set when it is either build.
+float crossing_limit(double L);
+// Whether launch_ingest takes the batch kernel (which fills whole chunks).
+bool ingest_batched(const IngestParams& p);
+// Chunks [c0, c1] of every tile from slot-major to particle-major, in place.
+cudaError_t particle_major(float* slab, int64_t ncols, int64_t ring, int comps, int64_t c0, int64_t c1,
+                           cudaStream_t st);
+// The FP32 builds of the per-call ingest kernel (common and precise-phase ring, without and
+// with sub-cycling); a kernel function pointer compares equal to the set when it is one.
 struct IngestKernels {
-    const void* plain;
-    const void* precise;
+    const void* build[4];
 };
-inline bool operator==(const void* f, const IngestKernels& k) { return f == k.plain || f == k.precise; }
+inline bool operator==(const void* f, const IngestKernels& k)
+{
+    return f == k.build[0] || f == k.build[1] || f == k.build[2] || f == k.build[3];
+}
 IngestKernels ingest_kernel_ptr();
 
 // Stream a radiation context orders its work on (for in-library callers that

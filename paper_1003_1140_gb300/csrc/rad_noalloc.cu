@@ -209,7 +209,10 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     ip.n_steps = (int32_t)n_calls;
     ip.step0 = 0;
     ip.dt = dt;
+    ip.idt = 1.0 / dt;
+    ip.nsub = 1;
     ip.box_L = box_L;
+    ip.lim = crossing_limit(box_L);
     double* state = reinterpret_cast<double*>(B + o_state);
     ip.x_prev = state;
     ip.r_prev = state + 3 * ncols;
@@ -220,7 +223,8 @@ extern "C" int rad_spectrum_noalloc(const double* dirs, int32_t D, const double*
     ip.ncols = ncols;
     ip.ring = ring;
     ip.keep0 = 0;
-    ip.keep1 = S;
+    ip.turned = 1;
+    ip.keep1 = ring;
     ip.comps = kCompsPlain;
     ip.K = K;
     ip.nblk = nblk;
