@@ -141,7 +141,9 @@ typedef struct {
 /* Tuning knobs; zero-initialise for the defaults.  Set before the first step. */
 typedef struct {
     int32_t variant;       /* RAD_VARIANT_*; rad_get_options reports the engine in use,
-                              RAD_VARIANT_AUTO for the block-moment kernel   */
+                              RAD_VARIANT_AUTO for the block-moment kernel,
+                              which the automatic choice takes where w_max dt
+                              <= 54 (anchor_K 32 within the default budget)  */
     int32_t anchor_K;      /* FP32 path re-anchor interval: 8, 16 or 32 samples for
                               every frequency; 0 with the automatic kernel choice
                               or a phase budget in reserved[3]: the longest of 8,
@@ -163,7 +165,11 @@ typedef struct {
     int32_t check_inputs;  /* 1: flag non-finite x/u (RAD_ENAN at finalize)    */
     int32_t blocks_per_sm; /* 0 (auto), 2, 3 or 4: resident blocks per SM the FP32
                               kernel is built for (its register budget); 4
-                              frequencies per thread go with 4, 16 with 2    */
+                              frequencies per thread go with 4, 16 with 2.
+                              Setting this or freq_per_lane leaves the
+                              block-moment kernel, except to the values that
+                              rad_get_options reports for it (with
+                              RAD_VARIANT_AUTO: anchor_K 32, 8, 4)           */
     int32_t subcycle;      /* 0 or 1: none; n >= 2: n sub-samples per PIC sample
                               (Sec. 2.2 sub-cycling of the tracked particles):
                               u linear in time between the half-step states,

@@ -94,7 +94,7 @@ constexpr int kFT = 8, kPairs = kFT / 2;
 // 20 warps at 96 registers 3.56 / 6.58 / 7.88 (register pairs no longer line up: a third
 // more moves), 12 warps at 168 registers 3.01 / 5.72 / 8.03, 8-warp blocks 2.72 / 5.13 /
 // 7.62 (slower as soon as units of different cost share a block).
-constexpr int kWarps = 4, kBlocks = 4, kThreads = kWarps * 32;
+constexpr int kWarps = 4, kBlocks = kMomentBlocks, kThreads = kWarps * 32;
 constexpr int kMaxP = 12;    // moments per sub-block
 
 // Polynomials cos t = sum_j C_j (-t^2)^j, sin t = t sum_j S_j (-t^2)^j, leading

@@ -717,6 +717,11 @@ static int freeze(rad_ctx* c)
         if (c->opt.variant == RAD_VARIANT_MIX && c->opt.reserved[1] > 0) c->cfg.np = c->opt.reserved[1];
         c->cfg.coh = c->mode == RAD_COHERENT;
         c->cfg.mb = c->opt.blocks_per_sm ? c->opt.blocks_per_sm : 2;
+        // what rad_get_options reports of the block-moment kernel, handed back
+        const bool moments = c->opt.variant == RAD_VARIANT_AUTO && c->opt.anchor_K == 32 &&
+                             c->opt.reserved[3] == 0 && c->cfg.ft == 8 &&
+                             c->opt.freq_per_lane == 8 && c->cfg.mb == kMomentBlocks;
+        if (moments) c->cfg.mb = 2;
         if (c->cfg.ft == 16 && c->cfg.mb != 2)
             return fail(c, RAD_EINVAL, "16 frequencies per thread is built for 2 blocks per SM only");
         if (c->cfg.ft == 4 && (c->cfg.mb != 4 || c->cfg.np != 0))
@@ -753,9 +758,11 @@ static int freeze(rad_ctx* c)
             c->cfg.ft = 8;
             c->cfg.np = 0;
         }
-        // the automatic engine at the 32-sample anchors is the block-moment kernel
-        c->cfg.mom = !prec && !c->cfg.band && c->opt.variant == RAD_VARIANT_AUTO && c->K == 32 &&
-                     c->opt.reserved[3] == 0 && c->cfg.ft == 8 && c->cfg.mb == 2;
+        // the automatic engine at the 32-sample anchors is the block-moment kernel; options
+        // that fix a direct kernel's build leave it
+        c->cfg.mom = moments || (!prec && !c->cfg.band && c->opt.variant == RAD_VARIANT_AUTO &&
+                                 c->K == 32 && c->opt.reserved[3] == 0 && !c->opt.freq_per_lane &&
+                                 !c->opt.blocks_per_sm);
         // anchor positions: one FP32 hi/lo 3-vector per particle per K samples of the ring
         c->nblk = c->ring / c->K;
         if (!c->anc32) {
@@ -1786,7 +1793,7 @@ int rad_get_options(const rad_ctx* c, rad_options* o)
     if (c->frozen && c->precision == RAD_FP32_SPLIT) {
         o->anchor_K = c->cfg.K;
         o->freq_per_lane = c->cfg.ft;
-        o->blocks_per_sm = c->cfg.mb;
+        o->blocks_per_sm = c->cfg.mom ? kMomentBlocks : c->cfg.mb;
         o->variant = c->cfg.pm ? RAD_VARIANT_PRECISE
                      : c->cfg.mom ? RAD_VARIANT_AUTO
                                   : (c->cfg.np > 0 ? RAD_VARIANT_MIX : RAD_VARIANT_SFU);

@@ -363,6 +363,7 @@ struct Accum32Config {
     bool mom = false;    // block-moment kernel (the automatic choice): 8 frequencies per
                          // thread, K 32
 };
+constexpr int kMomentBlocks = 4;   // its resident blocks per SM
 bool accum32_moment(const Accum32Params* p, const Accum32Config& cfg, int grid,
                     cudaStream_t st, cudaError_t* err, int* nb);
 bool accum32_ft8_sfu(const Accum32Params* p, const Accum32Config& cfg, int grid,
