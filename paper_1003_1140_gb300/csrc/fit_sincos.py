@@ -1,5 +1,5 @@
-"""Fit the polynomials of the FP32 kernels: the FMA-pipe e^{i theta} of the MIX
-variant, and the cos / sin of the block-moment kernel (fit_moment).
+"""Fit the kernels' polynomials: the FMA-pipe e^{i theta} of the FP32 MIX variant, and
+the cos / sin of the block-moment kernels, FP32 (fit_moment) and FP64 (fit_moment64).
 
 Method (written from the mathematics, not from any library's code):
   * half-angle reduction: theta/2 = k pi + y, |y| <= pi/2 (Cody & Waite two-
@@ -15,6 +15,9 @@ the error of the complete float32 evaluation; the unit test re-runs the
 float32 emulation and checks the bound.
 """
 from __future__ import annotations
+
+import math
+from decimal import Decimal, localcontext
 
 import numpy as np
 
@@ -102,6 +105,87 @@ def fit_moment(x0, n):
     return np.stack(out, 1).reshape(-1).astype(np.float32), worst
 
 
+def dec_cos_sin(t):
+    """cos t and sin t of a Decimal to the context's precision, by their power series."""
+    out = []
+    for first, k in ((Decimal(1), 0), (t, 1)):
+        term, tot = first, first
+        while term and abs(term) > abs(tot) * Decimal(10) ** -45:
+            k += 2
+            term = -term * t * t / (k * (k - 1))
+            tot += term
+        out.append(tot)
+    return out
+
+
+def _dec_solve(A, b):
+    """Gaussian elimination with row pivoting."""
+    n = len(b)
+    M = [row[:] + [v] for row, v in zip(A, b)]
+    for i in range(n):
+        k = max(range(i, n), key=lambda r: abs(M[r][i]))
+        M[i], M[k] = M[k], M[i]
+        for r in range(i + 1, n):
+            f = M[r][i] / M[i][i]
+            M[r] = [x - f * y for x, y in zip(M[r], M[i])]
+    x = [Decimal(0)] * n
+    for i in reversed(range(n)):
+        x[i] = (M[i][n] - sum(M[i][k] * x[k] for k in range(i + 1, n))) / M[i][i]
+    return x
+
+
+def _dec_minimax(basis, target, refs, n_iter=12):
+    """Coefficients of the minimax fit on a grid: basis[i][k], target[i] at grid point i, a
+    Remez exchange from the points refs; the best of its steps (where the target is next to
+    a multiple of the basis the exchange can run out of sign changes)."""
+    m = len(basis[0])
+    best = None
+    for _ in range(n_iter):
+        coef = _dec_solve([basis[i] + [Decimal((-1) ** k)] for k, i in enumerate(refs)],
+                          [target[i] for i in refs])[:m]
+        err = [t - sum(c * v for c, v in zip(coef, row)) for t, row in zip(target, basis)]
+        worst = max(map(abs, err))
+        if best is None or worst < best[0]:
+            best = (worst, coef)
+        idx, cur = [], 0
+        for i in range(1, len(err)):              # the extremum of every run of one sign
+            if (err[i] > 0) != (err[cur] > 0):
+                idx.append(cur)
+                cur = i
+            elif abs(err[i]) > abs(err[cur]):
+                cur = i
+        idx.append(cur)
+        while len(idx) > m + 1:
+            idx.pop(0 if abs(err[idx[0]]) < abs(err[idx[-1]]) else -1)
+        if len(idx) < m + 1 or idx == refs:
+            break
+        refs = idx
+    return best[1]
+
+
+def fit_moment64(x0, n):
+    """fit_moment in 50 decimal digits for FP64 coefficients: the leading ones exactly 1, each
+    next one rounded to float64 and the rest fitted again.  Interleaved as there."""
+    with localcontext() as ctx:
+        ctx.prec = 50
+        npts = 600
+        xs = [Decimal(x0) * (Decimal(1) - Decimal(math.cos(math.pi * i / npts))) / 2
+              for i in range(1, npts + 1)]
+        cs = [dec_cos_sin(x) for x in xs]
+        out = []
+        for odd in (0, 1):
+            pw = [[x ** (2 * k + odd) for k in range(n)] for x in xs]
+            coef = [Decimal(1)]
+            for step in range(1, n):
+                m = n - step
+                target = [c[odd] - sum(a * v for a, v in zip(coef, row)) for c, row in zip(cs, pw)]
+                refs = [min(npts - 1, max(0, round(npts * (k + 1) / (m + 1)) - 1)) for k in range(m + 1)]
+                c = _dec_minimax([row[step:] for row in pw], target, refs)
+                coef.append(Decimal(float(c[0])))
+            out.append([abs(float(c)) for c in coef])
+        return [v for pair in zip(*out) for v in pair]
+
+
 PI_HI = np.float32(np.pi)
 PI_LO = np.float32(np.pi - float(PI_HI))
 INV_PI = np.float32(1.0 / np.pi)
@@ -148,3 +232,5 @@ if __name__ == "__main__":
     print("max |error| of e^{i theta}, |theta| <= 2000:", max_error(S, C))
     c, e = fit_moment(2.5, 6)
     print("moments, |t| <= 2.5:", ", ".join(f"{v:.9e}f" for v in c), "max error", e)
+    for x0, n in ((0.45, 6), (1.2, 8), (2.5, 10)):
+        print(f"FP64 moments, |t| <= {x0}:", ", ".join(map(repr, fit_moment64(x0, n))))

@@ -24,9 +24,11 @@
 //
 // Measured: 1024 electrons x 2000 samples x 256 omega in [0.1, 300], one direction,
 // 33.4 -> 13.3 ms per launch; 301 + 47 particles, 8 directions, 150 omega, coherent, three
-// windows 26.2 -> 6.8 ms.  Against an 80-bit evaluation (12 particles, omega to 1000, gamma 3 and 10) every quarter of the
-// spectrum is closer than with the sincos kernel (relative L2 1.6e-15 / 2.1e-14, was
-// 2.3e-15 / 2.9e-14).
+// windows 26.2 -> 6.8 ms.  Against an 80-bit evaluation (three draws each, relative L2, sincos
+// kernel / this one): 96 particles of gamma 3, 2000 samples, omega to 300 8.7e-16 / 6.7e-16; 48
+// summed coherently 4.4e-15 / 3.6e-15; 32, omega to 1000, 1.4e-15 / 1.2e-15, of gamma 10
+// 1.14e-14 / 7.3e-15.  (A 64-bit evaluation that forms w phi as one rounded product, as the
+// sincos kernel did, agrees better with that kernel than either does with the exact sum.)
 #include "rad_internal.cuh"
 
 namespace rad {
@@ -39,21 +41,21 @@ constexpr int kFirstOfTile = 1, kLastOfTile = 2, kFirstOfItem = 4, kLastOfItem =
 constexpr double kMagic = 6755399441055744.0;   // 1.5 * 2^52: x + kMagic - kMagic = rint(x)
 
 // cos t = sum_j C_j (-t^2)^j, sin t = t sum_j S_j (-t^2)^j (C_0, S_0, C_1, ...): minimax
-// fits, to 1.3e-16 with 12 terms on |t| <= 0.45, 3e-17 with 16 on 1.2, 1.4e-16 with 20
-// on 2.5.
+// fits (fit_sincos.py, fit_moment64), the larger error of the two 7.8e-17 with 12 terms on
+// |t| <= 0.45, 2.9e-17 with 16 on 1.2, 7.2e-17 with 20 on 2.5.
 __device__ const double g_coef64[3][kMaxP] = {
-    {1.0, 1.0, 0.4999999999999751, 0.16666666666666183, 0.041666666665231875,
-     0.008333333333141972, 0.0013888888586501258, 0.00019841269517198042, 2.480129920177559e-05,
-     2.75570524043038e-06, 2.743076305279894e-07, 2.494662730994068e-08, 0, 0, 0, 0, 0, 0, 0, 0},
-    {1.0, 1.0, 0.49999999999999767, 0.1666666666666662, 0.0416666666666324, 0.008333333333329045,
-     0.0013888888886983898, 0.00019841269839396627, 2.480158678140812e-05, 2.755731879001551e-06,
-     2.755724206431354e-07, 2.5052051333424482e-08, 2.0870411886095404e-09, 1.6054769217448092e-10,
-     1.1198542945666875e-11, 7.476922764732039e-13, 0, 0, 0, 0},
-    {1.0, 1.0, 0.4999999999999979, 0.16666666666666627, 0.04166666666665545, 0.008333333333331984,
-     0.0013888888888658891, 0.00019841269841055513, 2.48015872776248e-05, 2.7557319205284773e-06,
-     2.755731778947366e-07, 2.5052107404166922e-08, 2.0876704671782594e-09, 1.605901154252185e-10,
-     1.1469563252395525e-11, 7.646491811600006e-13, 4.763287816847204e-14, 2.802864700244281e-15,
-     1.438388844007278e-16, 7.601823467651374e-18}};
+    {1.0, 1.0, 0.4999999999999825, 0.16666666666666435, 0.04166666666544268, 0.008333333333200448,
+     0.0013888888610645155, 0.00019841269575805384, 2.480131122756528e-05, 2.7557078979925243e-06,
+     2.7432934213223533e-07, 2.4951101621670652e-08, 0, 0, 0, 0, 0, 0, 0, 0},
+    {1.0, 1.0, 0.4999999999999984, 0.16666666666666646, 0.04166666666663812, 0.008333333333330467,
+     0.0013888888887176297, 0.00019841269839798658, 2.4801586814436715e-05, 2.7557318850581163e-06,
+     2.755724509036157e-07, 2.505205633787126e-08, 2.087055278373164e-09, 1.6054983232036807e-10,
+     1.1201163601728481e-11, 7.480625978115661e-13, 0, 0, 0, 0},
+    {1.0, 1.0, 0.49999999999999856, 0.1666666666666665, 0.0416666666666574, 0.008333333333332454,
+     0.00138888888886841, 0.000198412698411059, 2.4801587279386724e-05, 2.7557319208323927e-06,
+     2.7557317861678203e-07, 2.5052107514794437e-08, 2.0876706458048e-09, 1.6059014026862612e-10,
+     1.146958949098133e-11, 7.646525529615967e-13, 4.7634984499532814e-14, 2.8031185637892373e-15,
+     1.4391004071714364e-16, 7.60997019323244e-18}};
 constexpr float kX0 = 0.45f, kX1 = 1.2f, kX2 = 2.5f;
 
 // The walk over (work unit, particle, chunk), advanced by lane 0 only; a unit is
