@@ -1013,14 +1013,18 @@ int rad_mlp_init(rad_mlp** out, const int32_t* widths, int32_t n_layers, int32_t
     MAL(m->loss, sizeof(double));
     MAL(m->loss_part, (size_t)device_sms() * kEpiWarps * sizeof(double));
     MAL(m->xin, (size_t)R * m->w[0] * 4);
-    // split-K scratch: the forward and input-gradient products are R rows wide
-    // (the weight gradient reduces over R itself and never splits)
+    // split-K scratch of the products that split: the forward and input-gradient products are
+    // R rows wide (the weight gradient reduces over R itself and never splits)
     size_t work = 0;
+    auto need = [&](int M, int N, int K) {
+        const int S = split_count(M, N, K);
+        if (S > 1) work = std::max(work, (size_t)S * M * N);
+    };
     for (int l = 0; l < n_layers; ++l) {
         const int in = m->w[l], outw = m->w[l + 1];
         for (int rows = 128; rows <= R; rows += 128) {
-            work = std::max(work, (size_t)split_count(rows, outw, in) * rows * outw);
-            if (l > 0) work = std::max(work, (size_t)split_count(rows, in, outw) * rows * in);
+            need(rows, outw, in);
+            if (l > 0) need(rows, in, outw);
         }
     }
     MAL(m->work, work * 4);
