@@ -46,8 +46,8 @@ METRIC = "G particle·step·ω·n updates/s, FP32 split vs FP64 GPU at ≤1e-4 r
 # workload scaled to 4096 particles (same samples, directions and omegas), valid while
 # the code (comments aside) of the kernel and of its work-list builder is the code that
 # was captured; traffic scales with the particle count.
-TRAFFIC_CAPTURE = {"sources_sha256": "15c5fb7ede08e6d5241bac913ebc793d260cba3f8a6628d9546c7fdfd709074c",
-                   "bytes_per_launch": 692.5e6, "particles": 4096}
+TRAFFIC_CAPTURE = {"sources_sha256": "ea10a26cdaa0875ce5d46bc884db06d332773721a7d8a5104079a2be242802ed",
+                   "bytes_per_launch": 692.4e6, "particles": 4096}
 UNIT = "G updates/s"
 # phase budget (rad per update) of the accuracy side-run: the upper decade of the
 # precision workload's grid (dt 0.05, w <= 1000) takes anchor blocks of 8 samples

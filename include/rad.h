@@ -76,7 +76,7 @@ extern "C" {
 #define RAD_COHERENT 1       /* S = 1/(4 pi^2) |sum_j q_j A_j|^2 */
 
 /* arithmetic of the accumulation */
-#define RAD_FP64 0           /* FP64 geometry, phase and sums; CUDA double sincos */
+#define RAD_FP64 0           /* FP64 geometry, phase, sines and sums */
 #define RAD_FP32_SPLIT 1     /* FP32 bulk; FP64 retarded-time anchor every K samples */
 
 /* sincos engine of the FP32 split path */

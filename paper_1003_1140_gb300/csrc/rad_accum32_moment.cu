@@ -34,8 +34,12 @@
 // Against the direct kernel (which the explicit variants still run): 8195 particles x 4096
 // samples x 8 directions x 1024 omega, ingest included, 125.0 -> 77.4 ms; 1024 x 2000 x 192 x
 // 2048 356 -> 221 ms; 1024 x 2000 x 12 x 64 3.49 -> 1.35 ms.  Issue slots 58% busy, the
-// special-function pipe 63-68%, FMA 42%: dependent chains of four warps per scheduler, and the
-// instruction cache, are what is left.
+// special-function pipe 65-69%, FMA 45%: dependent chains of four warps per scheduler, and the
+// instruction cache, are what is left.  Tried and slower: eight sub-blocks of four samples for
+// larger w h (dense map 225 -> 241 ms, shard 79.5 -> 87.1: 60 issue slots per sub-block against
+// 68 for its direct sums, and more code); moments for the lower slot of the first direct pair (dense
+// map 225 -> 267 ms); sines of one pair in four by polynomial (direct work 7.70 -> 7.25 ms, but
+// mixed work 2.6% slower).
 #include "rad_accum32.cuh"
 
 namespace rad {
