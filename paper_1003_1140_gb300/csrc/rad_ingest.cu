@@ -18,7 +18,7 @@
 //     would be ten 4-byte stores to as many sectors of the sample-innermost ring (181 us
 //     per call of 557,056 particles); the chunk that is being filled is slot-major
 //     instead, eight particles to a sector, and turned when a window closes (76 us, and
-//     6.6 us per call for turning it; 135 us with four FP64 divisions per call and
+//     7.2 us per call for turning it; 135 us with four FP64 divisions per call and
 //     particle and the slot-major ring of before).
 // Both split a launch in time when the particles alone leave the GPU idle: a later
 // segment's starting image count is the launch's initial count plus the integer
@@ -34,7 +34,9 @@ namespace rad {
 // count (its nearest periodic image is d - L rint(d / L)).  A particle that did
 // not cross the boundary has |d| <= L/2, where that is 0 exactly; only a
 // crossing pays for the FP64 division, which this GPU runs on its 1/64-rate
-// FP64 pipe.  Same value in every case.
+// FP64 pipe.  Same value in every case; NaN where the displacement is not finite (or
+// 2^30 boxes long): the particle's unwrapped position is lost from there on, whichever
+// kernel takes its later calls.
 __device__ __forceinline__ double image_jump(double d, double L, double half_L)
 {
     if (!(L > 0.0) || fabs(d) <= half_L) return 0.0;
@@ -876,8 +878,8 @@ static void tile_range(IngestParams& q)
 // blocks on each SM), also for a chunk it fills in part only, so the shortest batch that pays
 // grows with the tiles.  FP32, us per call, tile kernel / ingest_kernel: 8000 particles,
 // batches of 16 calls 2.15 / 2.02, 32 1.38 / 1.78; 20,000, 64 2.17 / 1.86, 128 1.80 / 1.78
-// (and 0.24 for turning the chunks); from about 40,000 particles on (512 calls 2.79 / 2.38 and
-// 0.47; 65,536 4.38 / 3.31 and 0.77) never.  FP64, where ingest_kernel's three reciprocal
+// (and 0.26 for turning the chunks); from about 40,000 particles on (512 calls 2.79 / 2.38 and
+// 0.52; 65,536 4.38 / 3.31 and 0.85) never.  FP64, where ingest_kernel's three reciprocal
 // square roots per sample cost most: 65,536, 16 calls 17.8 / 13.2, 32 12.4 / 12.9, 512
 // 7.4 / 12.2.  Launches that may not leave slot-major chunks behind take the tile kernel
 // from 8 calls on.
